@@ -17,6 +17,7 @@
 #include <mutex>
 #include <vector>
 
+#include "cluster.h"
 #include "dispatch.h"
 #include "solver.cuh"
 
@@ -250,6 +251,37 @@ int batched_impl(const nvd_graph_t *gs, int32_t G, const int32_t *k_per, const v
     }
     const size_t szv = o.mode == NVD_MODE_FP64 ? 8 : 4;
     const size_t xsz = xdt == NVD_F64 ? 8 : 4;
+    if (o.mode == NVD_MODE_FP64 && !o.kt && !(o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION))) {
+        // one cluster per (graph, component, pair) where that is faster (cluster.cu)
+        ClusterPlan *cpl = nullptr;
+        NVD_TRY(cluster_plan_for(U, kmax, KT, (kmax + KT - 1) / KT, &cpl));
+        if (cpl) {
+            int wst = NVD_OK;
+            Owner *d_own = (Owner *)U->wsp("owners", (size_t)G * sizeof(Owner), &wst);
+            if (wst) return wst;
+            std::vector<Owner> own(G);
+            std::vector<int64_t> off(G + 1, 0);
+            for (int i = 0; i < G; ++i) {
+                own[i] = Owner{x[i], y[i], nullptr, u->node_off[i], gs[i]->n, k_per[i], u->seg_off[i], u->seg_off[i + 1], 0};
+                off[i + 1] = off[i] + k_per[i];
+            }
+            NVD_TRY_CUDA(cudaMemcpyAsync(d_own, own.data(), G * sizeof(Owner), cudaMemcpyHostToDevice, s));
+            ColResult *res = nullptr;
+            NVD_TRY(cluster_solve(U, cpl, o, d_own, own[0], G, kmax, xdt, false, nullptr, true, &res, s));
+            int overall = NVD_OK;
+            for (int i = 0; i < G; ++i)
+                for (int j = 0; j < k_per[i]; ++j) {
+                    const ColResult &r = res[(size_t)i * kmax + j];
+                    d2_out[off[i] + j] = r.d2;
+                    if (r.status != NVD_OK && overall != NVD_ERR_NUMERIC) overall = r.status;
+                    if (stats)
+                        stats[off[i] + j] = nvd_solve_stats{
+                            r.iters, 0, r.rr0 > 0.0 ? std::sqrt(std::max(r.rr, 0.0) / r.rr0) : 0.0, r.status, 0};
+                }
+            if (overall != NVD_OK) set_error("nvd_ge_distance_batched: some pair ended with status %d", overall);
+            return overall;
+        }
+    }
     Plan *pl = nullptr;
     NVD_TRY(get_plan(U, KT, (int)szv, (int)szv, &pl, false));   // the persistent kernel's register-path SpMM
     Ctx c;

@@ -103,6 +103,9 @@ struct Plan {
 namespace nvd {
 struct ElimState;   // exact low-degree elimination (elim.cu)
 void elim_state_delete(ElimState *e);
+struct ClusterState;   // one-cluster-per-pair solves (cluster.cu)
+void cluster_state_delete(ClusterState *c);
+int64_t cluster_state_bytes(const ClusterState *c);
 }  // namespace nvd
 
 struct nvd_graph_s {
@@ -139,6 +142,8 @@ struct nvd_graph_s {
     cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_used[2] = {nullptr, nullptr};
     // degree-1/2 nodes eliminated exactly and the reduced graph (nvd_graph_eliminate)
     std::unique_ptr<nvd::ElimState, void (*)(nvd::ElimState *)> elim{nullptr, nvd::elim_state_delete};
+    // plans of the one-cluster-per-pair solve (small and mid-sized graphs, FP64)
+    std::unique_ptr<nvd::ClusterState, void (*)(nvd::ClusterState *)> clusters{nullptr, nvd::cluster_state_delete};
     ~nvd_graph_s();
 
     void *wsp(const std::string &name, size_t bytes, int *st);

@@ -12,6 +12,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "cluster.h"
 #include "dispatch.h"
 #include "solver.cuh"
 
@@ -82,6 +83,61 @@ int check_opts(const nvd_solve_opts &o) {
     return NVD_OK;
 }
 
+// One cluster per (component, pair) instead of tiles over the whole graph (cluster.cu):
+// FP64, when the call leaves the form of the solve open (no tile width, persistent or
+// folded form, here or from the tuner, which times tiles), starts from zero and is not
+// being profiled launch by launch; cluster_plan_for then compares the two forms' times.
+// Host inputs are staged whole, so only up to 256 MB of them.
+int pick_cluster(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size_t in_bytes, bool warm,
+                 ClusterPlan **out) {
+    *out = nullptr;
+    if (o.mode != NVD_MODE_FP64 || o.kt || warm || prof_enabled() || g->tuned_kt[o.mode] ||
+        g->tuned_persistent[o.mode] ||
+        (o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION | NVD_SOLVE_TEST_TIMEOUT)) ||
+        ((o.flags & NVD_SOLVE_HOST_INPUTS) && 2 * in_bytes > ((size_t)1 << 28)))
+        return NVD_OK;
+    return cluster_plan_for(g, k, KT, (k + KT - 1) / KT, out);
+}
+
+// nvd_ge_distance through cluster_solve; arguments as in distance_impl.
+int cluster_distance(nvd_graph_t g, ClusterPlan *pl, const nvd_solve_opts &o, int32_t k, const void *x, const void *y,
+                     int32_t xdt, double *d2_out, void *z_out, nvd_solve_stats *stats, cudaStream_t s, bool idx) {
+    const size_t xsz = xdt == NVD_F64 ? 8 : 4, bytes = (size_t)k * g->n * xsz;
+    const bool host_in = o.flags & NVD_SOLVE_HOST_INPUTS, d2_dev = o.flags & NVD_SOLVE_D2_DEVICE;
+    const bool want = !d2_dev || stats || host_in;
+    int st = NVD_OK;
+    void *z = z_out;
+    double *d2 = d2_dev ? d2_out : nullptr;
+    if (host_in) {
+        void *sx = g->wsp("stage_x", bytes, &st), *sy = g->wsp("stage_y", bytes, &st);
+        if (z_out) z = g->wsp("stage_z", bytes, &st);
+        if (st) return st;
+        NVD_TRY_CUDA(cudaMemcpyAsync(sx, x, bytes, cudaMemcpyHostToDevice, s));
+        NVD_TRY_CUDA(cudaMemcpyAsync(sy, y, bytes, cudaMemcpyHostToDevice, s));
+        x = sx;
+        y = sy;
+    }
+    if (z && g->n_singleton > 0) NVD_TRY_CUDA(cudaMemsetAsync(z, 0, bytes, s));
+    const Owner own{x, y, z, 0, g->n, k, 0, g->nseg, idx ? 1 : 0};
+    ColResult *res = nullptr;
+    NVD_TRY(cluster_solve(g, pl, o, nullptr, own, 1, k, xdt, z != nullptr, d2, want, &res, s));
+    if (host_in && z_out) NVD_TRY_CUDA(cudaMemcpyAsync(z_out, z, bytes, cudaMemcpyDeviceToHost, s));
+    if (!(o.flags & NVD_SOLVE_NO_SYNC) || want) NVD_TRY_CUDA(cudaStreamSynchronize(s));
+    int overall = NVD_OK;
+    if (want)
+        for (int32_t j = 0; j < k; ++j) {
+            const ColResult &r = res[j];
+            if (!d2_dev) d2_out[j] = r.d2;
+            if (r.status != NVD_OK && overall != NVD_ERR_NUMERIC) overall = r.status;
+            if (stats)
+                stats[j] = nvd_solve_stats{r.iters, 0, r.rr0 > 0.0 ? std::sqrt(std::max(r.rr, 0.0) / r.rr0) : 0.0,
+                                           r.status, 0};
+        }
+    if (overall != NVD_OK) set_error("nvd_ge_distance: some pair ended with status %d (%s)", overall,
+                                     nvd_status_string(overall));
+    return overall;
+}
+
 // idx: x, y are [k] device int32 node ids (indicator pairs e_x - e_y); the caller
 // has checked them; host inputs and device d^2 are not used (z_out, if given, is
 // [k][n] of xdt).
@@ -108,6 +164,11 @@ int distance_impl(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_
     }
     DeviceGuard guard(g->device);
     const int KT = pick_kt(g, o, k);
+    {
+        ClusterPlan *cpl = nullptr;
+        NVD_TRY(pick_cluster(g, o, k, KT, (size_t)k * g->n * (xdt == NVD_F64 ? 8 : 4), z0 != nullptr, &cpl));
+        if (cpl) return cluster_distance(g, cpl, o, k, x, y, xdt, d2_out, z_out, stats, s, idx);
+    }
     const bool mixed = o.mode == NVD_MODE_MIXED;
     const size_t szv = o.mode == NVD_MODE_FP64 ? 8 : 4;
     const size_t xsz = xdt == NVD_F64 ? 8 : 4;
