@@ -194,7 +194,8 @@ void nvd_solve_opts_default(nvd_solve_opts *o);
 typedef struct {
     int32_t kt;            /* chosen right-hand sides per tile */
     int32_t row_max_pct;   /* light-row limit in percent of the default (50, 100 or 200) */
-    int32_t blocks_pct;    /* light CTA blocks per SpMV in percent of the default */
+    int32_t blocks_pct;    /* light CTA blocks per SpMV in percent of the default, one wave of four
+                              per SM (below 100: as 100) */
     int32_t persistent;    /* 1: one persistent launch per tile was faster */
     int32_t candidates;    /* configurations timed */
     int32_t fold_direction; /* 1: two kernels per iteration (NVD_SOLVE_FOLD_DIRECTION) were faster */

@@ -36,11 +36,16 @@ constexpr double d2_safety() { return 0.03; }
 constexpr int sp_vec(int KT, int szv) { return KT * szv >= 16 ? 16 / szv : KT; }
 constexpr int sp_lanes_per_row(int KT, int szv) { return KT / sp_vec(KT, szv); }
 constexpr int sp_slice_rows(int KT, int szv) { return 32 / sp_lanes_per_row(KT, szv); }
-// doubles of reduction scratch per CTA (KT = 1: every thread's partial of up to 4
-// sums, added by one warp per sum)
-constexpr int red_doubles(int KT) {
-    return KT == 1 ? 4 * NT : (NWARP * 4 * KT) > 256 ? NWARP * 4 * KT : 256;
-}
+// Longest row that one lane group of a multi-column SpMM takes (FP64 vectors); a longer
+// light row is a slice of its own, its entries dealt to the warp's lane groups.  A lane
+// group has two gathers in flight, about 400 clocks an entry, so a row of 1,000 entries (the
+// light-row limit at 4 columns) alone took 0.3 ms of a 0.33 ms iteration on a BA graph of
+// 60,000 nodes.  FP32 rows keep one lane group: their sums' order is part of the FP32
+// results.
+constexpr int sp_group_max(int KT, int szv) { return KT > 1 && szv == 8 ? 32 : INT32_MAX; }
+// doubles of reduction scratch per CTA: every thread's partial of up to 4 sums (one column,
+// added by one warp per sum), or of the 4 columns a thread holds of one sum
+constexpr int red_doubles(int) { return 4 * NT; }
 constexpr int vec_smem_bytes(int KT) { return (red_doubles(KT) + 4 * KT) * 8; }
 // Stream plans of multi-column tiles (stream.cuh): light rows of at most
 // 256 / H entries (longer slices would unbalance the warps of a block), heavy rows cut

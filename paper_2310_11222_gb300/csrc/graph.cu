@@ -373,7 +373,7 @@ int run_components(nvd_graph_s *g, std::vector<int32_t> &root, cudaStream_t s) {
 
 }  // namespace
 
-int target_blocks(const nvd_graph_s *g) { return 2 * g->num_sms * 8; }
+int target_blocks(const nvd_graph_s *g) { return 4 * g->num_sms; }
 
 // ------------------------------------------------------------------ TMA tensor maps
 
@@ -454,14 +454,17 @@ __global__ void k_fill_slices(int64_t n_slices, int H, const int64_t *__restrict
         const int r = (int)(t % H);
         const int64_t base = sl_base[sl];
         const int64_t L = (sl_base[sl + 1] - base) / H;
-        const int32_t row = sl_row[t];
-        const int32_t pad = row >= 0 ? row : sl_row[sl * H];
+        const int32_t first = sl_row[sl * H];
+        const bool one = H > 1 && sl_row[sl * H + 1] == -2;   // one row over all lane groups
+        const int32_t row = one ? first : sl_row[t];
+        const int32_t pad = row >= 0 ? row : first;
         const int64_t e0 = row >= 0 ? rowptr[row] : 0;
         const int64_t d = row >= 0 ? rowptr[row + 1] - e0 : 0;
         for (int64_t j = 0; j < L; ++j) {
-            const bool in = j < d;
-            sl_col[base + j * H + r] = in ? colidx[e0 + j] : pad;
-            sl_w[base + j * H + r] = in ? (TWO)w[e0 + j] : (TWO)0;
+            const int64_t e = one ? j * H + r : j;
+            const bool in = e < d;
+            sl_col[base + j * H + r] = in ? colidx[e0 + e] : pad;
+            sl_w[base + j * H + r] = in ? (TWO)w[e0 + e] : (TWO)0;
         }
     }
 }
@@ -618,6 +621,7 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
     const int64_t LONG = sp_long_max(KT);
     const int64_t CH = tma ? sp_chunk_stream(KT, szv) : sp_chunk(KT, szv);
     const int H = sp_slice_rows(KT, szv);
+    const int64_t GMAX = tma ? INT64_MAX : sp_group_max(KT, szv);
     const std::vector<int64_t> &rp = g->h_rowptr;
     const int nseg = g->nseg;
 
@@ -670,9 +674,7 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
     // warp rounds (NWARP slices of H rows) of about `target` work (entries + rows);
     // inside a block the rows are sorted by length (longest first, ties by row) and
     // dealt into slices.  Heavy blocks follow their segment's light blocks.
-    // (stream plans: half as many, larger light blocks; their warps split a block's
-    // slices statically, which balances better on more work)
-    const int T = std::max(1, (tma ? target_blocks(g) / 2 : target_blocks(g)) * g->sp.blocks_pct / 100);
+    const int T = std::max(1, (tma ? 2 : 1) * target_blocks(g) * std::max(g->sp.blocks_pct, 100) / 100);
     const double target = ltot / T;
     // block sizes in whole slices (warps take a block's slices as they free up)
     const int64_t QR = (int64_t)H;
@@ -686,7 +688,13 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
         for (size_t q = 0; q < ord.size(); ++q) ord[q] = (int64_t)q;
         std::stable_sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) { return lens[x] > lens[y]; });
         const int64_t first = (int64_t)sl_base.size() - 1;
-        for (size_t q0 = 0; q0 < ord.size(); q0 += H) {
+        size_t q0 = 0;
+        for (; q0 < ord.size() && lens[ord[q0]] > GMAX; ++q0) {   // a row over all lane groups
+            sl_row.push_back((int32_t)rows[ord[q0]]);
+            sl_row.insert(sl_row.end(), H - 1, -2);
+            sl_base.push_back(sl_base.back() + (lens[ord[q0]] + H - 1) / H * H);
+        }
+        for (; q0 < ord.size(); q0 += H) {
             int64_t L = 0;
             for (int r = 0; r < H; ++r) {
                 const size_t q = q0 + r;

@@ -168,7 +168,21 @@ template <> struct DotOf<float> { typedef DFloat type; };
 __device__ __forceinline__ void dot_zero(double &d) { d = 0.0; }
 __device__ __forceinline__ void dot_zero(DFloat &d) { d.hi = 0.f; d.lo = 0.f; }
 __device__ __forceinline__ double dot_get(double d) { return d; }
-__device__ __forceinline__ double dot_get(const DFloat &d) { return (double)d.hi + (double)d.lo; }
+// (double)f with integer instructions where f is normal or zero: a conversion is an FP64-pipe
+// instruction (16 clocks per warp and SM), these are about two.
+__device__ __forceinline__ double f2d(float f) {
+    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    return m == 0 ? __hiloint2double((int)b, 0) : (double)f;
+}
+__device__ __forceinline__ double dot_get(const DFloat &d) { return f2d(d.hi) + f2d(d.lo); }
+// A stored weight in the accumulator type.
+template <class TA, class TW>
+__device__ __forceinline__ TA weight_as(TW w) {
+    if constexpr (sizeof(TA) == 8 && sizeof(TW) == 4) return f2d(w);
+    else return (TA)w;
+}
 __device__ __forceinline__ void dot_add(double &d, double a) { d += a; }
 __device__ __forceinline__ void dot_fma(double &d, double a, double b) { d = fma(a, b, d); }
 __device__ __forceinline__ void dot_add(DFloat &d, float a) {
@@ -199,8 +213,7 @@ __device__ __forceinline__ void dot_to_double(const D (&a)[ND][VEC], double (&o)
 
 // Block-wide per-column sums.  Thread t holds acc[d][v] for column
 // (t % CG) * VEC + v.  On return tot[d * KT + j] (shared) holds the block total,
-// summed in a fixed order (KT = 1: per lane over the warps, then a butterfly;
-// KT > 1: warp butterfly, then warps 0..7).
+// summed in a fixed order.
 template <int ND, int KT, int VEC>
 __device__ __forceinline__ void block_reduce_cols(double (&acc)[ND > 0 ? ND : 1][VEC], double *red,
                                                   double *tot) {
@@ -223,28 +236,40 @@ __device__ __forceinline__ void block_reduce_cols(double (&acc)[ND > 0 ? ND : 1]
         }
         __syncthreads();
     } else if constexpr (ND > 0) {
-        constexpr int CG = KT / VEC;
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        // several columns: the threads' values form [NT * VEC / KT][KT] in shared memory;
+        // each step halves them or better with full warps (a butterfly in every warp spends
+        // the same FP64 instruction on ever fewer values: 136 per block and sum at 8 FP32
+        // columns, 33 this way)
+        static_assert(ND <= 4 && VEC <= 4, "reduction scratch holds 4 values per thread");
+        const int t = threadIdx.x;
+        double s[ND];
 #pragma unroll
-        for (int off = CG; off < 32; off <<= 1)
+        for (int d = 0; d < ND; ++d) {
 #pragma unroll
-            for (int d = 0; d < ND; ++d)
+            for (int v = 0; v < VEC; ++v) red[t * VEC + v] = acc[d][v];
+            __syncthreads();
+            s[d] = red[t];
 #pragma unroll
-                for (int v = 0; v < VEC; ++v)
-                    acc[d][v] += __shfl_xor_sync(NVD_FULLMASK, acc[d][v], off);
-        if (lane < CG) {
+            for (int v = 1; v < VEC; ++v) s[d] += red[t + v * NT];
+            __syncthreads();
+        }
 #pragma unroll
-            for (int d = 0; d < ND; ++d)
-#pragma unroll
-                for (int v = 0; v < VEC; ++v) red[(warp * ND + d) * KT + lane * VEC + v] = acc[d][v];
+        for (int d = 0; d < ND; ++d) red[d * NT + t] = s[d];
+        __syncthreads();
+        double q = 0.0;
+        if (t < ND * 64) {
+            const double *r = red + (t >> 6) * NT + (t & 63);
+            q = (r[0] + r[64]) + (r[128] + r[192]);
         }
         __syncthreads();
-        if (threadIdx.x < ND * KT) {
-            const int d = threadIdx.x / KT, j = threadIdx.x % KT;
-            double s = 0.0;
+        if (t < ND * 64) red[t] = q;
+        __syncthreads();
+        if (t < ND * 32) {
+            const int d = t >> 5, l = t & 31;
+            q = red[d * 64 + l] + red[d * 64 + 32 + l];
 #pragma unroll
-            for (int w = 0; w < NWARP; ++w) s += red[(w * ND + d) * KT + j];
-            tot[threadIdx.x] = s;
+            for (int off = 16; off >= KT; off >>= 1) q += __shfl_xor_sync(NVD_FULLMASK, q, off);
+            if (l < KT) tot[d * KT + l] = q;
         }
         __syncthreads();
     }
@@ -332,18 +357,28 @@ __device__ __forceinline__ void block_sum_slots(const double *a, int64_t a0, int
     __syncthreads();
 }
 
+// After this block's writes: count its arrival; *last (shared) says to all threads whether it
+// was the last of n, whose reads then see the others' writes.  The block barriers order the
+// other threads' writes and reads around thread 0's fences (fences are cumulative); a fence
+// in every warp cost about a microsecond of a block.
+__device__ __forceinline__ void arrive_last(unsigned *count, int32_t n, int *last) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        *last = (atomicAdd(count, 1u) == (unsigned)(n - 1));
+        __threadfence();
+    }
+    __syncthreads();
+}
+
 // After this block's writes to a slot of group [f, f + m): count the arrival; the
 // group's last writer adds the group into gpart at f.  Returns (block-uniformly)
 // whether this block did.
 template <int ND, int KT>
 __device__ __forceinline__ bool group_arrive(const Ctx &c, int64_t f, int32_t m, double *red) {
     __shared__ int s_glast;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_glast = (atomicAdd(&c.gcount[f], 1u) == (unsigned)(m - 1));
-    __syncthreads();
+    arrive_last(&c.gcount[f], m, &s_glast);
     if (!s_glast) return false;
-    __threadfence();
     block_sum_slots<ND, KT>(c.part, f, m, 1, nullptr, 0, 0, 0, c.part_stride, red);
     if (threadIdx.x < ND * KT) {
         const int d = threadIdx.x / KT, j = threadIdx.x % KT;
@@ -370,12 +405,8 @@ __device__ void seg_group_arrive(const Ctx &c, const Fin &fin, int seg, int64_t 
                                  int32_t hcnt, bool hgroup, double *red) {
     __shared__ int s_last;
     const int32_t ng = n_groups(cnt) + (hgroup ? n_groups(hcnt) : 0);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(&c.counter[seg], 1u) == (unsigned)(ng - 1));
-    __syncthreads();
+    arrive_last(&c.counter[seg], ng, &s_last);
     if (!s_last) return;
-    __threadfence();
     if (hgroup)
         block_sum_slots<ND, KT>(c.gpart, s0, n_groups(cnt), SLOT_GROUP, c.gpart, h0, n_groups(hcnt), SLOT_GROUP,
                                 c.part_stride, red);
@@ -413,12 +444,8 @@ __device__ void seg_arrive(const Ctx &c, const Fin &fin, int seg, int64_t slot, 
         if (group_arrive<ND, KT>(c, f, m, red)) seg_group_arrive<ND, KT>(c, fin, seg, s0, cnt, h0, hcnt, hgroup, red);
         return;
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(&c.counter[seg], 1u) == (unsigned)(cnt - 1));
-    __syncthreads();
+    arrive_last(&c.counter[seg], cnt, &s_last);
     if (!s_last) return;
-    __threadfence();
     block_sum_slots<ND, KT>(c.part, s0, cnt, 1, c.part, h0, hcnt, 1, c.part_stride, red);
     if (threadIdx.x < KT) {
         double v[ND];
@@ -796,7 +823,7 @@ __device__ __forceinline__ void spmm_chunk(const Ctx &c, const Epi &epi, int seg
             const int cc[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                if (eb + q >= it.e0 && eb + q < it.e1) s += (TA)w4[q] * (TA)LD::ld(src + cc[q]);
+                if (eb + q >= it.e0 && eb + q < it.e1) s += weight_as<TA>(w4[q]) * (TA)LD::ld(src + cc[q]);
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(NVD_FULLMASK, s, off);
@@ -826,7 +853,7 @@ __device__ __forceinline__ void spmm_chunk(const Ctx &c, const Epi &epi, int seg
             for (int u = 0; u < U; ++u)
                 if (e + u * S < it.e1) {
                     ca[u] = __ldcs(c.colidx + e + u * S);
-                    wa[u] = (TA)__ldcs(w + e + u * S);
+                    wa[u] = weight_as<TA>(__ldcs(w + e + u * S));
                 }
 #pragma unroll
             for (int u = 0; u < U; ++u)
@@ -855,13 +882,8 @@ __device__ __forceinline__ void spmm_chunk(const Ctx &c, const Epi &epi, int seg
     __syncthreads();
     __shared__ int s_fin;
     if (threadIdx.x < KT) c.hsum[(int64_t)(it.hbase + it.hchunk) * KT + threadIdx.x] = chunk[threadIdx.x];
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0)
-        s_fin = (atomicAdd(c.hcount + it.hrow, 1) == it.nchunk - 1);
-    __syncthreads();
+    arrive_last(reinterpret_cast<unsigned *>(c.hcount + it.hrow), it.nchunk, &s_fin);
     if (s_fin) {
-        __threadfence();
         if (threadIdx.x < KT) {
             double t = 0.0;
             for (int q = 0; q < it.nchunk; ++q)
@@ -913,10 +935,10 @@ __device__ __noinline__ void spmv1_long(const Ctx &c, const Epi &epi_in, int seg
             ld4_stream(w + qb, wq);
             const bool in0 = qb >= it.e0 && qb < it.e1, in1 = qb + 1 >= it.e0 && qb + 1 < it.e1;
             const bool in2 = qb + 2 >= it.e0 && qb + 2 < it.e1, in3 = qb + 3 >= it.e0 && qb + 3 < it.e1;
-            if (in0) s0 += (TA)wq[0] * (TA)LD::ld(src + cq.x);
-            if (in1) s1 += (TA)wq[1] * (TA)LD::ld(src + cq.y);
-            if (in2) s2 += (TA)wq[2] * (TA)LD::ld(src + cq.z);
-            if (in3) s3 += (TA)wq[3] * (TA)LD::ld(src + cq.w);
+            if (in0) s0 += weight_as<TA>(wq[0]) * (TA)LD::ld(src + cq.x);
+            if (in1) s1 += weight_as<TA>(wq[1]) * (TA)LD::ld(src + cq.y);
+            if (in2) s2 += weight_as<TA>(wq[2]) * (TA)LD::ld(src + cq.z);
+            if (in3) s3 += weight_as<TA>(wq[3]) * (TA)LD::ld(src + cq.w);
         }
         TA sum = (s0 + s1) + (s2 + s3);
 #pragma unroll
@@ -1038,7 +1060,7 @@ __device__ void spmv1_block(const Ctx &c, const Epi &epi, const TV *__restrict__
                         if (j + u < L) pv[u] = LD::ld(src + cu[u]);
 #pragma unroll
                     for (int u = 0; u < U; ++u)
-                        if (j + u < L) acc += (TA)wu[u] * (TA)pv[u];
+                        if (j + u < L) acc += weight_as<TA>(wu[u]) * (TA)pv[u];
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         cu[u] = cn[u];
@@ -1080,6 +1102,17 @@ __device__ void spmv1_block(const Ctx &c, const Epi &epi, const TV *__restrict__
         const int32_t hcnt = c.seg_heavy_off[seg + 1] - c.seg_heavy_off[seg];
         seg_arrive<ND, 1>(c, epi.fin, seg, b, tot, s0, cnt, h0, hcnt, red);
     }
+}
+
+// A slice that holds one row over all lane groups (sp_group_max; marked by row id -2 in every
+// group but the first): the groups' sums added into the first.
+template <int LPR, class TA, int VEC>
+__device__ __forceinline__ void warp_row_sum(int32_t i, TA (&acc)[VEC]) {
+    if (__shfl_sync(NVD_FULLMASK, i, 31) != -2) return;
+#pragma unroll
+    for (int off = LPR; off < 32; off <<= 1)
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) acc[v] += __shfl_xor_sync(NVD_FULLMASK, acc[v], off);
 }
 
 // A warp's fixed run of light slices [s_lo, s_hi) of a multi-column SpMM (tiles
@@ -1168,7 +1201,7 @@ __device__ __forceinline__ void spmm_light_run(const Ctx &c, Epi &e, const TV *_
                 const bool lo = ob + u * G < 32;
                 const int sl_lane = (ob + u * G + gid) & 31;
                 cu[u] = __shfl_sync(NVD_FULLMASK, lo ? mc : nc, sl_lane);
-                wu[u] = (TA)__shfl_sync(NVD_FULLMASK, lo ? mw : nw, sl_lane);
+                wu[u] = weight_as<TA>(__shfl_sync(NVD_FULLMASK, lo ? mw : nw, sl_lane));
             }
 #pragma unroll
             for (int u = 0; u < U; ++u)
@@ -1179,6 +1212,7 @@ __device__ __forceinline__ void spmm_light_run(const Ctx &c, Epi &e, const TV *_
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) acc[v] += wu[u] * (TA)pv[u][v];
         }
+        if constexpr (sp_group_max(KT, sizeof(TV)) != INT32_MAX) warp_row_sum<LPR>(i, acc);
         if (i >= 0) e.template elem<TV, TA, VEC>(c, i, col0, KT, own, acc, dg, dst, dot);
         base = nb;
         nb = nb2;
@@ -1255,7 +1289,7 @@ __device__ void spmm_block(const Ctx &c, const Epi &epi, const TV *__restrict__ 
                     for (int u = 0; u < U; ++u)
                         if (j + u < L) {
                             cu[u] = __ldcs(cp + (j + u) * G);
-                            wu[u] = (TA)__ldcs(wp + (j + u) * G);
+                            wu[u] = weight_as<TA>(__ldcs(wp + (j + u) * G));
                         }
 #pragma unroll
                     for (int u = 0; u < U; ++u)
@@ -1266,6 +1300,7 @@ __device__ void spmm_block(const Ctx &c, const Epi &epi, const TV *__restrict__ 
 #pragma unroll
                             for (int v = 0; v < VEC; ++v) acc[v] += wu[u] * (TA)pv[u][v];
                 }
+                if constexpr (sp_group_max(KT, sizeof(TV)) != INT32_MAX) warp_row_sum<LPR>(i, acc);
                 if (i >= 0) e.template elem<TV, TA, VEC>(c, i, col0, KT, own, acc, dg, dst, dot);
             }
         } else {

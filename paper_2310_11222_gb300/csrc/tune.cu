@@ -188,10 +188,9 @@ int tune_impl(nvd_graph_s *g, int32_t mode, int32_t k, uint32_t flags, nvd_tune_
     //    back, twice each, and the candidate must win by 2%: single timings differ
     //    by a few percent from run to run)
     for (int pass = 0; pass < 2; ++pass) {
-        // fewer, larger blocks (25%) balance the fixed warp runs of multi-column
-        // tiles better, and at four CTAs per SM fill one wave of 608 blocks
-        std::vector<int> pcts = {50, 200};
-        if (pass == 1 && best_kt > 1) pcts.insert(pcts.begin(), 25);
+        // row limit: half and twice the default; blocks: two waves instead of one
+        std::vector<int> pcts = {200};
+        if (pass == 0) pcts.insert(pcts.begin(), 50);
         for (int pct : pcts) {
             SpParams cand = g->sp;
             (pass == 0 ? cand.row_max_pct : cand.blocks_pct) = pct;
