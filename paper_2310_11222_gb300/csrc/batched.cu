@@ -254,7 +254,10 @@ int batched_impl(const nvd_graph_t *gs, int32_t G, const int32_t *k_per, const v
     if (o.mode == NVD_MODE_FP64 && !o.kt && !(o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION))) {
         // one cluster per (graph, component, pair) where that is faster (cluster.cu)
         ClusterPlan *cpl = nullptr;
-        NVD_TRY(cluster_plan_for(U, kmax, KT, (kmax + KT - 1) / KT, &cpl));
+        int cs = 0;
+        double us = 0.0;
+        NVD_TRY(cluster_estimate(U, kmax, &cs, &us));
+        if (cs && us <= tiles_iter_us(U->n, U->nnz, KT, (kmax + KT - 1) / KT)) NVD_TRY(cluster_plan_get(U, cs, &cpl));
         if (cpl) {
             int wst = NVD_OK;
             Owner *d_own = (Owner *)U->wsp("owners", (size_t)G * sizeof(Owner), &wst);

@@ -37,6 +37,7 @@
 
 #include "cluster.h"
 #include "dispatch.h"
+#include "onchip.cuh"
 
 namespace nvd {
 
@@ -44,6 +45,8 @@ void note_launch(int64_t n);
 int allow_dynamic_smem(const void *kern, int bytes);
 
 namespace {
+
+using namespace onchip;
 
 constexpr int CL_MAX_CS = 16;
 constexpr int CL_MAX_NT = 1024;
@@ -55,28 +58,16 @@ struct ClSeg {
     int64_t slot0;
     int32_t seg, n, spc, cta0, owner, pad;
 };
-// A CTA's share: items [item0, item0 + nitem) and their entries [e0, e0 + ne).
+// A CTA's share: items [item0, item0 + nitem) (32 lane groups of one lane) and their entries
+// [e0, e0 + ne).
 struct ClCta {
     int64_t item0, e0;
     int32_t nitem, ne;
 };
-// One warp's rows: `steps` steps of 32 entries from e (relative to the CTA's first), stored
-// in groups of 4 steps so that a lane reads its 4 columns with one 16-byte load and its 4
-// weights with two; lane l works for local slot slot + (l >> lg).
-struct ClItem {
-    int32_t e, steps, slot, lg;
-};
-// Place of step t of lane l relative to the item's first entry: columns [group][lane][4],
-// weights [group][2][lane][2] (16-byte accesses of neighbouring lanes are contiguous).
-__host__ __device__ constexpr int64_t cl_col_at(int64_t t, int l) { return (t >> 2) * 128 + l * 4 + (t & 3); }
-__host__ __device__ constexpr int64_t cl_w_at(int64_t t, int l) {
-    return (t >> 2) * 128 + ((t >> 1) & 1) * 64 + l * 2 + (t & 1);
-}
-
 struct ClArgs {
     const ClSeg *segs;
     const ClCta *ctas;
-    const ClItem *items;
+    const Item *items;
     const int32_t *col;        // slots, relative to the component's first
     const double *w;
     const int32_t *node;       // slot -> user node (-1: empty)
@@ -124,17 +115,6 @@ struct ClState {
     double cred[2][2][CL_MAX_CS * CL_RW];   // [parity][sum][rank * CL_RW + warp]: partial sums of all CTAs
     double irho;
 };
-
-// Tests on the bits: a comparison is an FP64 instruction too.
-__device__ __forceinline__ bool finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
-__device__ __forceinline__ bool pos_finite(double v) {
-    return __double_as_longlong(v) > 0 && finite(v);
-}
-
-__device__ __forceinline__ double butterfly(double v, int width) {
-    for (int off = width / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
 
 // Sum v0 (and v1) over the cluster.  Every thread's value goes through shared memory to
 // CL_RW warps per sum, which add them lane by lane, then by a butterfly; their totals go to
@@ -213,10 +193,10 @@ __global__ void __launch_bounds__(CL_MAX_NT, 1) k_cluster_pcg(const __grid_const
     double *red = pall + (PG ? spc : cs * spc);
     const double *deg = a.deg + slot0, *dinv = a.dinv + slot0, *wv = a.w + ct.e0;
     const int32_t *cv = a.col + ct.e0;
-    const ClItem *items = a.items + ct.item0;
+    const Item *items = a.items + ct.item0;
     if constexpr (MS) {
         double *sd = red + 2 * nt, *sdi = sd + (ONE ? 0 : spc), *sw = sdi + (ONE ? 0 : spc);
-        ClItem *si = reinterpret_cast<ClItem *>(sw + ct.ne);          // ne is a multiple of 32
+        Item *si = reinterpret_cast<Item *>(sw + ct.ne);          // ne is a multiple of 32
         int32_t *sc = reinterpret_cast<int32_t *>(si + ct.nitem);
         if constexpr (!ONE) {
             for (int s = tid; s < spc; s += nt) {
@@ -342,7 +322,7 @@ __global__ void __launch_bounds__(CL_MAX_NT, 1) k_cluster_pcg(const __grid_const
         // next beta off the chain)
         if (tid == nt - 1) st.irho = 1.0 / st.rho;
         for (int i = warp; i < ct.nitem; i += nw) {
-            const ClItem it = items[i];
+            const Item it = items[i];
             const int4 *cp = reinterpret_cast<const int4 *>(cv + it.e) + lane;
             const double2 *wp = reinterpret_cast<const double2 *>(wv + it.e) + lane;
             const int L = it.steps;
@@ -512,35 +492,6 @@ __global__ void k_cluster_collect(const ColResult *__restrict__ part, const Owne
     res[t] = r;
 }
 
-// Entries of the plan from the CSR, one warp per slot: entry j of a row with g lanes from
-// lane l0 on is step j / g of lane l0 + j % g of its item (slot_g: g | l0 << 8), padding has
-// weight 0 on the row's own slot.  Also the slot's degree and its inverse.
-template <class TW>
-__global__ void k_cluster_fill(int64_t n_slots, const int32_t *__restrict__ slot_row, const int64_t *__restrict__ slot_e,
-                               const int32_t *__restrict__ slot_len, const int32_t *__restrict__ slot_g,
-                               const int32_t *__restrict__ slot_of, const int32_t *__restrict__ slot_rel,
-                               const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-                               const TW *__restrict__ w, const double *__restrict__ deg64,
-                               const double *__restrict__ dinv64, int32_t *col, double *wo, double *deg, double *dinv) {
-    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n_slots; t += nwarp) {
-        const int32_t row = slot_row[t], L = slot_len[t], g = slot_g[t] & 255, l0 = slot_g[t] >> 8;
-        const int64_t e0 = row >= 0 ? rowptr[row] : 0;
-        const int64_t d = row >= 0 ? rowptr[row + 1] - e0 : 0;
-        for (int64_t j = lane; j < L; j += 32) {
-            const bool in = j < d;
-            const int l = l0 + (int)(j % g);
-            col[slot_e[t] + cl_col_at(j / g, l)] = in ? slot_of[colidx[e0 + j]] : slot_rel[t];
-            wo[slot_e[t] + cl_w_at(j / g, l)] = in ? (double)w[e0 + j] : 0.0;
-        }
-        if (lane == 0) {
-            deg[t] = row >= 0 ? deg64[row] : 0.0;
-            dinv[t] = row >= 0 ? dinv64[row] : 0.0;
-        }
-    }
-}
-
 struct ClClass {
     int cs = 1, nt = 128;
     bool pg = false, ms = false, l2 = false, one = false;
@@ -556,12 +507,13 @@ struct ClusterPlan {
     std::vector<ClClass> classes;
     int64_t n_slots = 0, n_entries = 0;
     DevBuf segs, ctas, items, col, w, node, deg, dinv;
-    DevBuf slot_row, slot_e, slot_len, slot_g, slot_of, slot_rel;   // what k_cluster_fill needs (weight updates)
+    DevBuf tasks, slot_row, slot_of;   // what the weight updates need
+    int64_t n_tasks = 0;
 };
 
 struct ClusterState {
     std::map<int, std::unique_ptr<ClusterPlan>> plans;   // by cs_max
-    int64_t max_n = -1, max_nnz = 0, max_deg = 0;        // largest component
+    int64_t max_n = -1, max_nnz = 0, rows = 0;           // largest component, all components
     ColResult *h_res = nullptr;                          // pinned read-back
     size_t h_cap = 0;
     ~ClusterState() {
@@ -575,9 +527,8 @@ int64_t cluster_state_bytes(const ClusterState *c) {
     if (c)
         for (auto &kv : c->plans)
             for (const DevBuf *d : {&kv.second->segs, &kv.second->ctas, &kv.second->items, &kv.second->col,
-                                    &kv.second->w, &kv.second->node, &kv.second->deg,
-                                    &kv.second->dinv, &kv.second->slot_row, &kv.second->slot_e, &kv.second->slot_len,
-                                    &kv.second->slot_g, &kv.second->slot_of, &kv.second->slot_rel})
+                                    &kv.second->w, &kv.second->node, &kv.second->deg, &kv.second->dinv,
+                                    &kv.second->tasks, &kv.second->slot_row, &kv.second->slot_of})
                 b += (int64_t)d->bytes;
     return b;
 }
@@ -591,7 +542,7 @@ size_t cl_smem(int cs, int64_t spc, int nt, bool pg) {
 }
 // More shared memory: the degrees, their inverses, ne entries and the items of a CTA.
 size_t cl_smem_matrix(int64_t spc, int nt, int64_t ne, int64_t items) {
-    return (spc <= nt ? 0 : (size_t)spc * 16) + (size_t)ne * 12 + (size_t)items * sizeof(ClItem);
+    return (spc <= nt ? 0 : (size_t)spc * 16) + (size_t)ne * 12 + (size_t)items * sizeof(Item);
 }
 // Longest row that keeps one lane, and 4 lanes.  With few rows per CTA an item is one
 // serial chain of multiply-adds (65 clocks each) that sets the pace, so rows are split
@@ -606,20 +557,8 @@ ClLimits cl_limits(int64_t rows_per_cta) {
 int64_t cl_spc_estimate(int64_t n, int cs) { return ((n + cs - 1) / cs + 31) / 32 * 32 + 64; }
 
 int fill_cluster_plan(nvd_graph_s *g, ClusterPlan *pl, cudaStream_t s) {
-    if (pl->n_slots == 0) return NVD_OK;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((pl->n_slots + 7) / 8, (int64_t)g->num_sms * 16));
-    auto go = [&](auto *w) {
-        k_cluster_fill<<<grid, 256, 0, s>>>(pl->n_slots, pl->slot_row.as<int32_t>(), pl->slot_e.as<int64_t>(),
-                                            pl->slot_len.as<int32_t>(), pl->slot_g.as<int32_t>(),
-                                            pl->slot_of.as<int32_t>(), pl->slot_rel.as<int32_t>(), g->rowptr.as<int64_t>(),
-                                            g->colidx.as<int32_t>(), w, g->deg64.as<double>(),
-                                            g->dinv64.as<double>(), pl->col.as<int32_t>(), pl->w.as<double>(),
-                                            pl->deg.as<double>(), pl->dinv.as<double>());
-    };
-    if (g->wdtype == NVD_F64) go(g->w.as<double>());
-    else go(g->w.as<float>());
-    NVD_TRY_CUDA(cudaGetLastError());
-    return NVD_OK;
+    return fill_onchip(g, pl->n_tasks, 32, pl->tasks, pl->slot_of, pl->col, pl->w, pl->n_slots, pl->slot_row, pl->deg,
+                       pl->dinv, s);
 }
 
 // CTAs per cluster of a component of n rows when the largest uses cs_max: enough for
@@ -650,9 +589,9 @@ int build_cluster_plan(nvd_graph_s *g, int cs_max, ClusterPlan **out) {
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return rows_of(a) > rows_of(b); });
     std::vector<ClSeg> segs;
     std::vector<ClCta> ctas;
-    std::vector<ClItem> items;
-    std::vector<int64_t> slot_e;
-    std::vector<int32_t> node, slot_row, slot_len, slot_g, slot_rel, slot_of(g->n, 0);
+    std::vector<Item> items;
+    std::vector<FillTask> tasks;
+    std::vector<int32_t> node, slot_row, slot_of(g->n, 0);
     std::vector<int32_t> rows, cnt;
     int64_t ne = 0;
     for (int s : order) {
@@ -712,10 +651,6 @@ int build_cluster_plan(nvd_graph_s *g, int cs_max, ClusterPlan **out) {
         segs.push_back(sg);
         const size_t base = slot_row.size();
         slot_row.resize(base + cs * spc, -1);
-        slot_e.resize(base + cs * spc, 0);
-        slot_len.resize(base + cs * spc, 0);
-        slot_g.resize(base + cs * spc, 1);
-        slot_rel.resize(base + cs * spc, 0);
         node.resize(base + cs * spc, -1);
         for (int c = 0; c < cs; ++c) {
             ClCta ct{};
@@ -726,17 +661,17 @@ int build_cluster_plan(nvd_graph_s *g, int cs_max, ClusterPlan **out) {
                 const int g1 = todo[i].second;
                 const int64_t r0 = todo[i].first, steps = (len_of(rows[r0]) + g1 - 1) / g1;
                 const int64_t room = std::max<int64_t>((steps + 3) / 4 * 4, 4);   // whole groups
-                items.push_back(ClItem{(int32_t)(ne - ct.e0), (int32_t)steps, slot, g1 == 32 ? 5 : g1 == 4 ? 2 : 0});
+                items.push_back(Item{(int32_t)(ne - ct.e0), (int32_t)steps, slot, g1 == 32 ? 5 : g1 == 4 ? 2 : 0});
                 for (int l = 0; l < 32 / g1; ++l, ++slot) {
                     const size_t t = base + (size_t)c * spc + slot;
-                    const int32_t row = r0 + l < n ? rows[r0 + l] : -1;
+                    const int32_t self = (int32_t)((int64_t)c * spc + slot);
+                    const bool in = r0 + l < n;
+                    const int32_t row = in ? rows[r0 + l] : -1;
                     slot_row[t] = row;
-                    slot_e[t] = ne;
-                    slot_len[t] = (int32_t)(room * g1);
-                    slot_g[t] = g1 | (l * g1) << 8;
-                    slot_rel[t] = (int32_t)((int64_t)c * spc + slot);
-                    if (row >= 0) {
-                        slot_of[row] = slot_rel[t];
+                    tasks.push_back(FillTask{ne, in ? rp[row] : 0, in ? (int32_t)len_of(row) : 0, (int32_t)(room * g1),
+                                             g1 | (l * g1) << 8, self});
+                    if (in) {
+                        slot_of[row] = self;
                         node[t] = perm.empty() ? row : perm[row];
                     }
                 }
@@ -776,13 +711,11 @@ int build_cluster_plan(nvd_graph_s *g, int cs_max, ClusterPlan **out) {
     };
     NVD_TRY(up(pl->segs, segs.data(), segs.size() * sizeof(ClSeg)));
     NVD_TRY(up(pl->ctas, ctas.data(), ctas.size() * sizeof(ClCta)));
-    NVD_TRY(up(pl->items, items.data(), items.size() * sizeof(ClItem)));
+    NVD_TRY(up(pl->items, items.data(), items.size() * sizeof(Item)));
     NVD_TRY(up(pl->node, node.data(), node.size() * 4));
     NVD_TRY(up(pl->slot_row, slot_row.data(), slot_row.size() * 4));
-    NVD_TRY(up(pl->slot_e, slot_e.data(), slot_e.size() * 8));
-    NVD_TRY(up(pl->slot_len, slot_len.data(), slot_len.size() * 4));
-    NVD_TRY(up(pl->slot_g, slot_g.data(), slot_g.size() * 4));
-    NVD_TRY(up(pl->slot_rel, slot_rel.data(), slot_rel.size() * 4));
+    pl->n_tasks = (int64_t)tasks.size();
+    NVD_TRY(up(pl->tasks, tasks.data(), tasks.size() * sizeof(FillTask)));
     NVD_TRY(up(pl->slot_of, slot_of.data(), slot_of.size() * 4));
     NVD_TRY(pl->deg.alloc(std::max<int64_t>(pl->n_slots, 1) * 8));
     NVD_TRY(pl->dinv.alloc(std::max<int64_t>(pl->n_slots, 1) * 8));
@@ -858,8 +791,8 @@ double cl_iter_us(int64_t n, int64_t nnz, int cs, bool pg, int m) {
 
 }  // namespace
 
-int cluster_plan_for(nvd_graph_s *g, int64_t cols, int gen_kt, int gen_tiles, ClusterPlan **out) {
-    *out = nullptr;
+int cluster_estimate(nvd_graph_s *g, int64_t cols, int *cs_out, double *us_out) {
+    *cs_out = 0;
     if (g->nseg < 1 || cols < 1) return NVD_OK;
     if (!g->clusters) g->clusters.reset(new ClusterState());
     ClusterState *cst = g->clusters.get();
@@ -867,6 +800,7 @@ int cluster_plan_for(nvd_graph_s *g, int64_t cols, int gen_kt, int gen_tiles, Cl
         cst->max_n = 0;
         for (int s = 0; s < g->nseg; ++s) {
             const int64_t n = g->h_seg_end[s] - g->h_seg_begin[s];
+            cst->rows += n;
             cst->max_n = std::max(cst->max_n, n);
             cst->max_nnz = std::max(cst->max_nnz, g->h_rowptr[g->h_seg_end[s]] - g->h_rowptr[g->h_seg_begin[s]]);
         }
@@ -875,40 +809,38 @@ int cluster_plan_for(nvd_graph_s *g, int64_t cols, int gen_kt, int gen_tiles, Cl
     if (4 * 8 * cl_spc_estimate(cst->max_n, CL_MAX_CS) > room) return NVD_OK;
     ClusterLimits lim;
     NVD_TRY(cluster_limits(g, &lim));
-    // total rows and entries, for the share of small components
-    int64_t rows = 0, nnz = g->nnz;
-    for (int s = 0; s < g->nseg; ++s) rows += g->h_seg_end[s] - g->h_seg_begin[s];
-    // the largest component's tasks decide the cluster size: least (waves x iteration time)
+    // the largest component's tasks decide the cluster size: least (waves x iteration time),
+    // all tasks as if they had its size, as many as the rows make
+    const double tasks = std::max<double>((double)cols, (double)cols * cst->rows / std::max<int64_t>(cst->max_n, 1));
     double best = 1e300;
-    int best_cs = 0;
     for (int k = 0; k < 5; ++k) {
         const int cs = 1 << k;
         if (!lim.fit[k]) continue;
         const int64_t spc = cl_spc_estimate(cst->max_n, cs);
         const bool pg = cl_smem(cs, spc, CL_MAX_NT, false) > CL_SMEM_MAX;
         if (pg && 4 * 8 * spc > room) continue;
-        // all tasks as if they had the largest component's size, scaled by the rows
-        const double tasks = std::max<double>((double)cols, (double)cols * rows / std::max<int64_t>(cst->max_n, 1));
         const int nt = cl_threads(spc);
         const int m = (int)std::min<int64_t>(CL_MAX_NT / nt, (int64_t)(CL_SMEM_MAX / (cl_smem(cs, spc, nt, pg) + 2048)));
-        const double it = cl_iter_us(cst->max_n, cst->max_nnz, cs, pg, m);
-        const double t = std::ceil(tasks / ((double)lim.fit[k] * std::max(m, 1))) * it;
+        const double t = std::ceil(tasks / ((double)lim.fit[k] * std::max(m, 1))) *
+                         cl_iter_us(cst->max_n, cst->max_nnz, cs, pg, m);
         if (t < best) {
             best = t;
-            best_cs = cs;
+            *cs_out = cs;
         }
     }
-    if (!best_cs) return NVD_OK;
-    // the host-driven loop: three launches per iteration and tile, and 3.2 times the tile's
-    // FP64 instructions (measured: 108 us for 16 columns of 30,000 rows, 90 us for 8 of 100,000)
-    const double gen = gen_tiles * (22.0 + 3.2 * gen_kt * ((double)nnz + 10.0 * (double)rows) / 6.3e5);
-    if (best > gen) return NVD_OK;
-    auto &slot = cst->plans[best_cs];
+    *us_out = best;
+    return NVD_OK;
+}
+
+int cluster_plan_get(nvd_graph_s *g, int cs, ClusterPlan **out) {
+    *out = nullptr;
+    ClusterState *cst = g->clusters.get();
+    auto &slot = cst->plans[cs];
     if (!slot) {
         ClusterPlan *p = nullptr;
-        const int rc = build_cluster_plan(g, best_cs, &p);
+        const int rc = build_cluster_plan(g, cs, &p);
         if (rc != NVD_OK) {
-            cst->plans.erase(best_cs);
+            cst->plans.erase(cs);
             return rc;
         }
         slot.reset(p);
@@ -949,7 +881,7 @@ int cluster_solve(nvd_graph_s *g, ClusterPlan *pl, const nvd_solve_opts &o, cons
             ClArgs a{};
             a.segs = pl->segs.as<ClSeg>() + cl.seg0;
             a.ctas = pl->ctas.as<ClCta>();
-            a.items = pl->items.as<ClItem>();
+            a.items = pl->items.as<Item>();
             a.col = pl->col.as<int32_t>();
             a.w = pl->w.as<double>();
             a.node = pl->node.as<int32_t>();

@@ -7,10 +7,18 @@ namespace nvd {
 
 struct ClusterPlan;
 
-// Plan for solving `cols` columns per component with one cluster each, or *out = NULL
-// where the components do not fit or the host-driven loop (gen_tiles tiles of gen_kt
-// columns) is estimated to be faster.
-int cluster_plan_for(nvd_graph_s *g, int64_t cols, int gen_kt, int gen_tiles, ClusterPlan **out);
+// Estimated microseconds of one iteration of `cols` columns per component with one cluster
+// each, and the cluster size that takes them; *cs = 0 where the components do not fit.
+int cluster_estimate(nvd_graph_s *g, int64_t cols, int *cs, double *us);
+// The plan for that cluster size (after cluster_estimate), or *out = NULL if it does not fit.
+int cluster_plan_get(nvd_graph_s *g, int cs, ClusterPlan **out);
+// Estimated microseconds of one iteration of the host-driven loop on `tiles` tiles of kt FP64
+// columns, fitted to runs from 3 * 10^4 to 10^6 rows: three launches and their block reductions,
+// and 1.4 times the FP64 instructions (a multiply-add per entry and 10 operations per row, at 2
+// lanes per SM and clock).
+inline double tiles_iter_us(int64_t n, int64_t nnz, int kt, int tiles) {
+    return tiles * (32.0 + 2.0 * kt + 1.4 * kt * ((double)nnz + 10.0 * (double)n) / 6.3e5);
+}
 
 // Solve K columns for every owner (owners_dev: device table of n_owner, or NULL: own0);
 // the owners' x, y, z point at column 0 and hold kc columns.  d2dev: [K] device, one

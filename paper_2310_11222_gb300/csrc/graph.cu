@@ -21,6 +21,7 @@
 
 #include "cluster.h"
 #include "graph.h"
+#include "resident.h"
 
 namespace nvd {
 
@@ -941,7 +942,7 @@ int64_t nvd_graph_s::device_bytes() const {
                                      &kv.second->sl_wsplit, &kv.second->sl_wrun})
             b += (int64_t)d->bytes;
     for (auto &kv : ws) b += (int64_t)kv.second->bytes;
-    return b + nvd::cluster_state_bytes(clusters.get());
+    return b + nvd::cluster_state_bytes(clusters.get()) + nvd::resident_state_bytes(resident.get());
 }
 
 // ------------------------------------------------------------------ C ABI
@@ -1284,6 +1285,7 @@ static int set_weights_impl(nvd_graph_t g, const void *w, int32_t wdtype, uint32
     }
     for (auto &kv : g->plans) NVD_TRY(fill_plan_slices(g, kv.second.get(), s));
     NVD_TRY(cluster_refill(g, s));
+    NVD_TRY(resident_refill(g, s));
     NVD_TRY_CUDA(cudaStreamSynchronize(s));
     g->elim.reset();            // the reduced graph depends on the weights
     g->id = next_graph_id();    // caches keyed by the handle (batched unions, captured launches) miss

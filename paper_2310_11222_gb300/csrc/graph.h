@@ -106,6 +106,9 @@ void elim_state_delete(ElimState *e);
 struct ClusterState;   // one-cluster-per-pair solves (cluster.cu)
 void cluster_state_delete(ClusterState *c);
 int64_t cluster_state_bytes(const ClusterState *c);
+struct ResidentState;  // one-kernel solves with the vectors on chip (resident.cu)
+void resident_state_delete(ResidentState *c);
+int64_t resident_state_bytes(const ResidentState *c);
 }  // namespace nvd
 
 struct nvd_graph_s {
@@ -144,6 +147,8 @@ struct nvd_graph_s {
     std::unique_ptr<nvd::ElimState, void (*)(nvd::ElimState *)> elim{nullptr, nvd::elim_state_delete};
     // plans of the one-cluster-per-pair solve (small and mid-sized graphs, FP64)
     std::unique_ptr<nvd::ClusterState, void (*)(nvd::ClusterState *)> clusters{nullptr, nvd::cluster_state_delete};
+    // plans of the solve with the vectors on chip (one component, FP64)
+    std::unique_ptr<nvd::ResidentState, void (*)(nvd::ResidentState *)> resident{nullptr, nvd::resident_state_delete};
     ~nvd_graph_s();
 
     void *wsp(const std::string &name, size_t bytes, int *st);

@@ -14,6 +14,7 @@
 
 #include "cluster.h"
 #include "dispatch.h"
+#include "resident.h"
 #include "solver.cuh"
 
 using namespace nvd;
@@ -83,28 +84,49 @@ int check_opts(const nvd_solve_opts &o) {
     return NVD_OK;
 }
 
-// One cluster per (component, pair) instead of tiles over the whole graph (cluster.cu):
-// FP64, when the call leaves the form of the solve open (no tile width, persistent or
-// folded form, here or from the tuner, which times tiles), starts from zero and is not
-// being profiled launch by launch; cluster_plan_for then compares the two forms' times.
-// Host inputs are staged whole, so only up to 256 MB of them.
-int pick_cluster(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size_t in_bytes, bool warm,
-                 ClusterPlan **out) {
-    *out = nullptr;
+// Which form an FP64 solve takes when the call leaves it open: no tile width, persistent or
+// folded form, here or from the tuner (which times tiles), a start from zero and no
+// launch-by-launch profiling.  Three estimates of one iteration over all k columns decide:
+// one cluster per (component, pair) (cluster.cu), one persistent kernel with the vectors on
+// chip (resident.cu, the tile width of the least time), the host-driven tiles.  Host inputs
+// of the on-chip forms are staged whole, so only up to 256 MB of them.
+int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size_t in_bytes, bool warm,
+                ClusterPlan **cluster, ResidentPlan **resident) {
+    *cluster = nullptr;
+    *resident = nullptr;
     if (o.mode != NVD_MODE_FP64 || o.kt || warm || prof_enabled() || g->tuned_kt[o.mode] ||
-        g->tuned_persistent[o.mode] ||
+        g->tuned_persistent[o.mode] || g->tuned_fold[o.mode] ||
         (o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION | NVD_SOLVE_TEST_TIMEOUT)) ||
         ((o.flags & NVD_SOLVE_HOST_INPUTS) && 2 * in_bytes > ((size_t)1 << 28)))
         return NVD_OK;
-    return cluster_plan_for(g, k, KT, (k + KT - 1) / KT, out);
+    double best = tiles_iter_us(g->n, g->nnz, KT, (k + KT - 1) / KT), us = 0.0;
+    int cs = 0, rkt = 0;
+    NVD_TRY(cluster_estimate(g, k, &cs, &us));
+    if (cs && us < best) best = us;
+    else cs = 0;
+    // a call without a final synchronisation has nobody to report a wait that gave up to
+    if (g->nseg == 1 && !(o.flags & NVD_SOLVE_NO_SYNC))
+        for (int kt : {1, 4, 8, 16}) {
+            if (kt > KT && kt > 1) break;
+            us = ((k + kt - 1) / kt) * resident_iter_us(g->h_seg_end[0] - g->h_seg_begin[0], g->nnz, kt);
+            ResidentPlan *pl = nullptr;
+            if (us < best) NVD_TRY(resident_plan_for(g, kt, &pl));
+            if (pl) {
+                best = us;
+                rkt = kt;
+                *resident = pl;
+            }
+        }
+    if (!rkt && cs) NVD_TRY(cluster_plan_get(g, cs, cluster));
+    return NVD_OK;
 }
 
-// nvd_ge_distance through cluster_solve; arguments as in distance_impl.
-int cluster_distance(nvd_graph_t g, ClusterPlan *pl, const nvd_solve_opts &o, int32_t k, const void *x, const void *y,
+// nvd_ge_distance through cluster_solve or resident_solve; arguments as in distance_impl.
+int onchip_distance(nvd_graph_t g, ClusterPlan *cpl, ResidentPlan *rpl, const nvd_solve_opts &o, int32_t k, const void *x, const void *y,
                      int32_t xdt, double *d2_out, void *z_out, nvd_solve_stats *stats, cudaStream_t s, bool idx) {
     const size_t xsz = xdt == NVD_F64 ? 8 : 4, bytes = (size_t)k * g->n * xsz;
     const bool host_in = o.flags & NVD_SOLVE_HOST_INPUTS, d2_dev = o.flags & NVD_SOLVE_D2_DEVICE;
-    const bool want = !d2_dev || stats || host_in;
+    const bool want = !d2_dev || stats || host_in || rpl;
     int st = NVD_OK;
     void *z = z_out;
     double *d2 = d2_dev ? d2_out : nullptr;
@@ -120,7 +142,8 @@ int cluster_distance(nvd_graph_t g, ClusterPlan *pl, const nvd_solve_opts &o, in
     if (z && g->n_singleton > 0) NVD_TRY_CUDA(cudaMemsetAsync(z, 0, bytes, s));
     const Owner own{x, y, z, 0, g->n, k, 0, g->nseg, idx ? 1 : 0};
     ColResult *res = nullptr;
-    NVD_TRY(cluster_solve(g, pl, o, nullptr, own, 1, k, xdt, z != nullptr, d2, want, &res, s));
+    if (rpl) NVD_TRY(resident_solve(g, rpl, o, own, k, xdt, d2, want, &res, s));
+    else NVD_TRY(cluster_solve(g, cpl, o, nullptr, own, 1, k, xdt, z != nullptr, d2, want, &res, s));
     if (host_in && z_out) NVD_TRY_CUDA(cudaMemcpyAsync(z_out, z, bytes, cudaMemcpyDeviceToHost, s));
     if (!(o.flags & NVD_SOLVE_NO_SYNC) || want) NVD_TRY_CUDA(cudaStreamSynchronize(s));
     int overall = NVD_OK;
@@ -166,8 +189,9 @@ int distance_impl(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_
     const int KT = pick_kt(g, o, k);
     {
         ClusterPlan *cpl = nullptr;
-        NVD_TRY(pick_cluster(g, o, k, KT, (size_t)k * g->n * (xdt == NVD_F64 ? 8 : 4), z0 != nullptr, &cpl));
-        if (cpl) return cluster_distance(g, cpl, o, k, x, y, xdt, d2_out, z_out, stats, s, idx);
+        ResidentPlan *rpl = nullptr;
+        NVD_TRY(pick_onchip(g, o, k, KT, (size_t)k * g->n * (xdt == NVD_F64 ? 8 : 4), z0 != nullptr, &cpl, &rpl));
+        if (cpl || rpl) return onchip_distance(g, cpl, rpl, o, k, x, y, xdt, d2_out, z_out, stats, s, idx);
     }
     const bool mixed = o.mode == NVD_MODE_MIXED;
     const size_t szv = o.mode == NVD_MODE_FP64 ? 8 : 4;
