@@ -8,11 +8,13 @@
 // W_sym = (W + W^T)/2.  The two stored entries of an undirected edge thus sum to
 // -(z_u - z_v)^2, the derivative with respect to the edge weight.
 //
-// The weight gradient is an edge gather over the CSR: z is first laid out as
-// [n][KT] tiles (one 16-byte aligned row per node) so each stored entry reads one
-// contiguous row of its neighbour, like the SpMM.
+// The weight gradient is a gather over the undirected edges: z is first laid out as
+// [n][KT] tiles (one 16-byte aligned row per node); an edge reads its two nodes' rows and
+// writes its two stored entries, which have the same derivative.  The edge list (its nodes
+// and the places of its entries) is made from the CSR once per handle.
 #include <algorithm>
 #include <cstring>
+#include <utility>
 
 #include "graph.h"
 #include "kernels.cuh"
@@ -45,47 +47,134 @@ __global__ void k_z_tile(const TZ *__restrict__ z, int64_t n, int k, int c0, con
     }
 }
 
-// One warp per row u: for every stored entry e = (u, v),
-//   g[e] (+)= -1/2 sum_j gbar_j (zt[u][j] - zt[v][j])^2.
-template <class TZ, class TG, int KT, bool ACC>
-__global__ void __launch_bounds__(256) k_grad_edges(int64_t n, const int64_t *__restrict__ rowptr,
-                                                    const int32_t *__restrict__ colidx,
-                                                    const TZ *__restrict__ zt, const double *__restrict__ gb,
-                                                    TG *__restrict__ g) {
-    constexpr int VEC = dev::VecCfg<TZ, KT>::VEC, LPR = KT / VEC, G = 32 / LPR;
-    const int lane = threadIdx.x & 31;
-    const int gi = lane / LPR, sub = lane % LPR, col0 = sub * VEC;
-    double gbl[VEC];
+// The edge list from the CSR: one edge for every stored entry (u, v), u < v, with the place of
+// (v, u) beside its own (rev; -1 if it is not stored), and one for every entry u > v whose
+// mirror is not stored (a pattern the caller vouched for).  A block takes 256 rows, a warp a
+// row at a time: once to count, then (WRITE), with the block's range of the list reserved, to write.
+__device__ __forceinline__ int64_t find_entry(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                                              int32_t row, int32_t col) {
+    int64_t lo = __ldg(rowptr + row), hi = __ldg(rowptr + row + 1);
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (__ldg(colidx + mid) < col) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo < __ldg(rowptr + row + 1) && __ldg(colidx + lo) == col ? lo : -1;
+}
+template <bool WRITE>
+__global__ void __launch_bounds__(256) k_edge_list(int64_t n, const int64_t *__restrict__ rowptr,
+                                                   const int32_t *__restrict__ colidx, bool symmetric,
+                                                   unsigned long long *total, int2 *__restrict__ uv,
+                                                   longlong2 *__restrict__ at) {
+    __shared__ unsigned cnt[256];
+    __shared__ unsigned long long base;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t r0 = (int64_t)blockIdx.x * 256; r0 < n; r0 += (int64_t)gridDim.x * 256) {
+        for (int pass = 0; pass < (WRITE ? 2 : 1); ++pass) {
+            for (int q = warp; q < 256 && r0 + q < n; q += 8) {
+                const int32_t u = (int32_t)(r0 + q);
+                const int64_t e0 = __ldg(rowptr + u), e1 = __ldg(rowptr + u + 1);
+                unsigned done = 0;
+                for (int64_t eb = e0; eb < e1; eb += 32) {
+                    const int64_t e = eb + lane;
+                    int32_t v = -1;
+                    int64_t rev = -1;
+                    bool take = false;
+                    if (e < e1) {
+                        v = __ldg(colidx + e);
+                        // counting needs only the mirrors of entries below the diagonal, and
+                        // those only where the pattern was not checked
+                        if (v > u ? WRITE && pass == 1 : !symmetric) rev = find_entry(rowptr, colidx, v, u);
+                        take = v > u || (!symmetric && rev < 0);
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, take);
+                    if (pass && take) {
+                        const unsigned long long o = base + cnt[q] + done + __popc(m & ((1u << lane) - 1u));
+                        uv[o] = make_int2(u, v);
+                        at[o] = make_longlong2(e, rev);
+                    }
+                    done += __popc(m);
+                }
+                if (!pass && lane == 0) cnt[q] = done;
+            }
+            __syncthreads();
+            if (!pass && warp == 0) {   // running sums of the 256 counts, 8 per lane
+                unsigned c[8], s = 0;
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) gbl[v] = gb[col0 + v];
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+                for (int q = 0; q < 8; ++q) {
+                    c[q] = r0 + lane * 8 + q < n ? cnt[lane * 8 + q] : 0u;
+                    s += c[q];
+                }
+                unsigned incl = s;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const unsigned o = __shfl_up_sync(0xffffffffu, incl, off);
+                    if (lane >= off) incl += o;
+                }
+                unsigned run = incl - s;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    cnt[lane * 8 + q] = run;
+                    run += c[q];
+                }
+                if (lane == 31) base = atomicAdd(total, (unsigned long long)incl);
+            }
+            __syncthreads();
+        }
+    }
+}
+
+template <class T> __device__ __forceinline__ double to_f64(T v) {
+    if constexpr (sizeof(T) == 4) return dev::f2d(v);
+    else return v;
+}
+
+// For every edge (u, v): g[entries of the edge] (+)= -1/2 sum_j gbar_j (zt[u][j] - zt[v][j])^2.
+// One lane per edge, two from 8 columns on, each taking every second 16 bytes of the rows.
+// Bound by the FP64 pipe: three operations per edge and column and, per 16 edges, one to add
+// the lane pair and one to scale.  A warp per row that took every stored entry with a lane group
+// per entry did each edge twice and spent 5 of 11 instructions on adding and scaling 4 entries
+// at 16 FP64 columns: 10^6 edges of a BA graph took 644 us, this way 106 us; 5 * 10^6 edges and 32
+// columns 4,824 us, this way 950 us.
+template <class TZ, class TG, int KT, bool ACC>
+__global__ void __launch_bounds__(256) k_grad_edges(int64_t n_edges, const int2 *__restrict__ uv,
+                                                    const longlong2 *__restrict__ at, const TZ *__restrict__ zt,
+                                                    const double *__restrict__ gb, TG *__restrict__ g) {
+    constexpr int VEC = dev::VecCfg<TZ, KT>::VEC, LPE = KT >= 8 ? 2 : 1, P = KT / (VEC * LPE);
+    static_assert(P >= 1, "columns fill the lanes");
+    const int lane = threadIdx.x & 31, sub = lane % LPE;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = warp; u < n; u += nw) {
-        const int64_t e0 = __ldg(rowptr + u), e1 = __ldg(rowptr + u + 1);
-        if (e0 == e1) continue;
-        TZ own[VEC];
-        dev::ldv<dev::LdRO, TZ, VEC>(zt + u * KT + col0, own);
-        for (int64_t eb = e0; eb < e1; eb += G) {
-            const int64_t e = eb + gi;
-            const bool ok = e < e1;
-            double s = 0.0;
-            if (ok) {
-                const int32_t v = __ldcs(colidx + e);
-                TZ zv[VEC];
-                dev::ldv<dev::LdRO, TZ, VEC>(zt + (int64_t)v * KT + col0, zv);
+    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b * (32 / LPE) < n_edges; b += nw) {
+        const int64_t e = b * (32 / LPE) + lane / LPE;
+        double s = 0.0;
+        longlong2 pos = make_longlong2(-1, -1);
+        if (e < n_edges) {
+            const int2 nd = __ldcs(uv + e);
+            pos = __ldcs(at + e);
+            const TZ *zu = zt + (int64_t)nd.x * KT, *zv = zt + (int64_t)nd.y * KT;
+#pragma unroll(P < 4 ? P : 4)
+            for (int i = 0; i < P; ++i) {
+                const int c0 = (i * LPE + sub) * VEC;
+                TZ a[VEC], c[VEC];
+                dev::ldv<dev::LdRO, TZ, VEC>(zu + c0, a);
+                dev::ldv<dev::LdRO, TZ, VEC>(zv + c0, c);
 #pragma unroll
                 for (int q = 0; q < VEC; ++q) {
-                    const double d = (double)own[q] - (double)zv[q];
-                    s += gbl[q] * d * d;
+                    const double d = to_f64(a[q]) - to_f64(c[q]);
+                    s += __ldg(gb + c0 + q) * d * d;
                 }
             }
-#pragma unroll
-            for (int off = 1; off < LPR; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            if (ok && sub == 0) {
-                const double val = -0.5 * s;
-                if (ACC) g[e] = (TG)((double)g[e] + val);
-                else g[e] = (TG)val;
-            }
+        }
+        if (LPE == 2) s += __shfl_xor_sync(0xffffffffu, s, 1);
+        const double val = -0.5 * s;
+        // two lanes: one entry each
+        if (sub == 0 && pos.x >= 0) {
+            if (ACC) g[pos.x] = (TG)((double)g[pos.x] + val);
+            else g[pos.x] = (TG)val;
+        }
+        if (sub == LPE - 1 && pos.y >= 0) {
+            if (ACC) g[pos.y] = (TG)((double)g[pos.y] + val);
+            else g[pos.y] = (TG)val;
         }
     }
 }
@@ -124,6 +213,35 @@ int grid_cap(int64_t work, int num_sms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)num_sms * 32));
 }
 
+// The handle's edge list, made on first use.
+int edge_list(nvd_graph_s *g, cudaStream_t s) {
+    if (g->grad_uv.p) return NVD_OK;
+    int st = NVD_OK;
+    unsigned long long *total = (unsigned long long *)g->wsp("grad_total", 8, &st);
+    if (st) return st;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((g->n + 255) / 256, (int64_t)g->num_sms * 8));
+    auto run = [&](auto kern, int2 *uv, longlong2 *at, unsigned long long *out) -> int {
+        NVD_TRY_CUDA(cudaMemsetAsync(total, 0, 8, s));
+        kern<<<grid, 256, 0, s>>>(g->n, g->rowptr.as<int64_t>(), g->colidx.as<int32_t>(), g->sym_checked, total, uv, at);
+        NVD_TRY_CUDA(cudaGetLastError());
+        NVD_TRY_CUDA(cudaMemcpyAsync(out, total, 8, cudaMemcpyDeviceToHost, s));
+        NVD_TRY_CUDA(cudaStreamSynchronize(s));
+        return NVD_OK;
+    };
+    unsigned long long ne = 0, written = 0;
+    NVD_TRY(run(k_edge_list<false>, nullptr, nullptr, &ne));
+    DevBuf uv, at;
+    NVD_TRY(uv.alloc((size_t)ne * sizeof(int2)));
+    NVD_TRY(at.alloc((size_t)ne * sizeof(longlong2)));
+    NVD_TRY(run(k_edge_list<true>, uv.as<int2>(), at.as<longlong2>(), &written));
+    std::swap(g->grad_uv.p, uv.p);
+    std::swap(g->grad_uv.bytes, uv.bytes);
+    std::swap(g->grad_at.p, at.p);
+    std::swap(g->grad_at.bytes, at.bytes);
+    g->grad_edges = (int64_t)ne;
+    return NVD_OK;
+}
+
 template <class TZ, class TW, int KT>
 int grad_w_impl(nvd_graph_s *g, int k, const TZ *z, const double *gbar, TW *grad_w, cudaStream_t s) {
     int st = NVD_OK;
@@ -140,19 +258,19 @@ int grad_w_impl(nvd_graph_s *g, int k, const TZ *z, const double *gbar, TW *grad
         if (st) return st;
     }
     const int zgrid = (int)((g->n + 31) / 32);
-    const int egrid = grid_cap(g->n * 32, g->num_sms);
+    NVD_TRY(edge_list(g, s));
+    const int64_t ne = g->grad_edges;
+    const int2 *uv = g->grad_uv.as<int2>();
+    const longlong2 *at = g->grad_at.as<longlong2>();
+    const int egrid = grid_cap(ne * (KT >= 8 ? 2 : 1), g->num_sms);
     for (int t = 0; t < ntile; ++t) {
         k_z_tile<TZ, KT><<<zgrid, 256, 0, s>>>(z, g->n, k, t * KT, g->perm.as<int32_t>(), zt);
-        if (direct) {
-            k_grad_edges<TZ, TW, KT, false><<<egrid, 256, 0, s>>>(g->n, g->rowptr.as<int64_t>(),
-                                                                   g->colidx.as<int32_t>(), zt, gbp, grad_w);
-        } else if (t == 0) {
-            k_grad_edges<TZ, double, KT, false><<<egrid, 256, 0, s>>>(
-                g->n, g->rowptr.as<int64_t>(), g->colidx.as<int32_t>(), zt, gbp + t * KT, gint);
-        } else {
-            k_grad_edges<TZ, double, KT, true><<<egrid, 256, 0, s>>>(
-                g->n, g->rowptr.as<int64_t>(), g->colidx.as<int32_t>(), zt, gbp + t * KT, gint);
-        }
+        if (direct)
+            k_grad_edges<TZ, TW, KT, false><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbp, grad_w);
+        else if (t == 0)
+            k_grad_edges<TZ, double, KT, false><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbp, gint);
+        else
+            k_grad_edges<TZ, double, KT, true><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbp + t * KT, gint);
         NVD_TRY_CUDA(cudaGetLastError());
     }
     if (!direct) {

@@ -932,7 +932,7 @@ void *nvd_graph_s::wsp(const std::string &name, size_t bytes, int *st) {
 int64_t nvd_graph_s::device_bytes() const {
     int64_t b = 0;
     for (const nvd::DevBuf *d : {&rowptr, &colidx, &w, &w32, &deg64, &dinv64, &deg32, &dinv32,
-                                 &perm, &uent, &seg_begin, &seg_end, &seg_owner})
+                                 &perm, &uent, &seg_begin, &seg_end, &seg_owner, &grad_uv, &grad_at})
         b += (int64_t)d->bytes;
     for (auto &kv : plans)
         for (const nvd::DevBuf *d : {&kv.second->items, &kv.second->sblk, &kv.second->vblk,
@@ -1047,6 +1047,7 @@ static int graph_create_impl(nvd_graph_t *out, int64_t n, int64_t nnz, const int
             set_error("nvd_graph_create: the CSR is not symmetric (structure or weights)");
             return NVD_ERR_NOT_SYMMETRIC;
         }
+        g->sym_checked = true;
     }
 
     // connected components; relabel if some component is not a contiguous range

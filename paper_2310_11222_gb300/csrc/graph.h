@@ -139,6 +139,10 @@ struct nvd_graph_s {
     int32_t tuned_fold[3] = {0, 0, 0};        // per solve mode: 1 = two kernels per iteration were faster
     std::map<int64_t, std::unique_ptr<nvd::Plan>> plans;
     std::map<std::string, std::unique_ptr<nvd::DevBuf>> ws;  // named lazily-grown workspace
+    // undirected edges for the weight gradient (built on first use): nodes, places of the two entries
+    nvd::DevBuf grad_uv, grad_at;
+    int64_t grad_edges = 0;
+    bool sym_checked = false;    // the pattern passed the symmetry check at creation
     // host-input staging: a copy stream and per-slot events (two slots), created on
     // first use, so the next tile's host-to-device copy overlaps the current solve
     cudaStream_t copy_stream = nullptr;
