@@ -561,12 +561,13 @@ int fill_cluster_plan(nvd_graph_s *g, ClusterPlan *pl, cudaStream_t s) {
                        pl->dinv, s);
 }
 
-// CTAs per cluster of a component of n rows when the largest uses cs_max: enough for
-// CL_ROWS rows per CTA (one warp per SM quarter).
-constexpr int64_t CL_ROWS = 128;
+// CTAs per cluster of a component of n rows when the largest uses cs_max: one up to 512 rows
+// (an iteration without cluster barriers takes 8,000 to 11,000 clocks, 4 CTAs took 11,600, and
+// components of one class run in one launch, not one class after another), else about 256
+// rows per CTA (2,000 rows: 8 and 16 CTAs the same).
 int cl_cs(int64_t n, int cs_max) {
     int cs = 1;
-    while (cs < cs_max && n > (int64_t)cs * CL_ROWS) cs *= 2;
+    while (n > 512 && cs < cs_max && n > (int64_t)cs * 256) cs *= 2;
     return cs;
 }
 
