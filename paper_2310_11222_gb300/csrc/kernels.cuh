@@ -359,14 +359,13 @@ __device__ __forceinline__ void block_sum_slots(const double *a, int64_t a0, int
 
 // After this block's writes: count its arrival; *last (shared) says to all threads whether it
 // was the last of n, whose reads then see the others' writes.  The block barriers order the
-// other threads' writes and reads around thread 0's fences (fences are cumulative); a fence
-// in every warp cost about a microsecond of a block.
+// other threads' writes and reads around thread 0's release and acquire, which are cumulative.
 __device__ __forceinline__ void arrive_last(unsigned *count, int32_t n, int *last) {
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        *last = (atomicAdd(count, 1u) == (unsigned)(n - 1));
-        __threadfence();
+        unsigned before;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(count) : "memory");
+        *last = before == (unsigned)(n - 1);
     }
     __syncthreads();
 }

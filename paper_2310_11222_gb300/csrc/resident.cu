@@ -100,7 +100,8 @@ __device__ __forceinline__ bool grid_meet(const RsArgs &a, RsState &st, unsigned
     target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
+        // release and acquire at GPU scope order the whole CTA's writes and reads through the
+        // block barriers around them
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
         unsigned seen;
         const uint64_t t0 = timer_ns();
@@ -113,7 +114,6 @@ __device__ __forceinline__ bool grid_meet(const RsArgs &a, RsState &st, unsigned
                 break;
             }
         }
-        __threadfence();
     }
     __syncthreads();
     return st.fail == 0;
