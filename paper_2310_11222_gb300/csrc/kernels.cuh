@@ -470,13 +470,21 @@ __device__ void heavy_arrive(const Ctx &c, const Fin &fin, int seg, int64_t hs, 
 }
 
 // Is any column of the segment still iterating?  (Constant during one phase:
-// only the segment's own finalizer changes it, after all its blocks arrived.)
+// only the segment's own finalizer changes it, after all its blocks arrived.)  Warp 0 reads,
+// a lane per column, for the whole block: every block of a pass asks the same few lines of L2,
+// which serve about one request a clock.  With every thread reading every column it was
+// 155,000 of them per pass over one segment: 32 FP32 columns of a power-law graph of 2 * 10^6
+// nodes (MIXED) took 80.2 ms, this way 70.5; 16 FP64 columns of a BA graph of 200,000 5.5 ms,
+// this way 4.8.
 template <int KT>
 __device__ __forceinline__ bool seg_live(const Ctx &c, int seg) {
-    int a = 0;
-#pragma unroll
-    for (int j = 0; j < KT; ++j) a |= __ldcg(c.active + (int64_t)seg * KT + j);
-    return a != 0;
+    __shared__ int s_live;
+    if (threadIdx.x < 32) {
+        const int any = __any_sync(NVD_FULLMASK, __ldcg(c.active + (int64_t)seg * KT + threadIdx.x % KT) != 0);
+        if (threadIdx.x == 0) s_live = any;
+    }
+    __syncthreads();
+    return s_live != 0;
 }
 
 // ------------------------------------------------------------------ finalizers

@@ -60,7 +60,10 @@ constexpr int persist_unroll() { return VecCfg<TV, KT>::VEC * (int)sizeof(TV) >=
 // less but ran slower: call overhead and saved registers on every block.)
 template <class TV, int KT, class Op, int U>
 __device__ __forceinline__ void vec_phase(const Ctx &c, const Op op, char *smem) {
-    for (int64_t b = blockIdx.x; b < c.n_vblk; b += gridDim.x) vec_block<TV, KT, Op, U>(c, op, b, smem);
+    for (int64_t b = blockIdx.x; b < c.n_vblk; b += gridDim.x) {
+        vec_block<TV, KT, Op, U>(c, op, b, smem);
+        __syncthreads();   // the next block's scalars reuse the shared memory these were read from
+    }
 }
 template <class TV, class TW, class TA, int KT, class Epi>
 __device__ __forceinline__ void spmm_phase(const Ctx &c, const Epi epi, const TV *src, TV *dst, char *smem) {

@@ -20,23 +20,31 @@ template <class Op, class = void> struct LiveOnStep { static constexpr bool valu
 template <class Op> struct LiveOnStep<Op, decltype((void)Op::LIVE_ON_STEP)> {
     static constexpr bool value = Op::LIVE_ON_STEP;
 };
-template <int KT>
-__device__ __forceinline__ bool seg_stepped(const Ctx &c, int seg) {
-    bool a = false;
-#pragma unroll
-    for (int j = 0; j < KT; ++j) a = a || __ldcg(c.alpha + (int64_t)seg * KT + j) != 0.0;
-    return a;
-}
+
+// The pass's per-column scalars (at most 3 per column, Op::stage) into shared memory and
+// whether the segment needs the pass: read once per block, by warp 0, for the reason given at
+// seg_live (single-RHS FP64 solves of 10^6 nodes 17.5 to 16.9 ms per 8 pairs; 1% or less at
+// several columns).  `sh` holds 4 * KT doubles.
 template <int KT, class Op>
-__device__ __forceinline__ bool op_live(const Ctx &c, int seg) {
-    if constexpr (LiveOnStep<Op>::value) return seg_stepped<KT>(c, seg);
-    else if constexpr (Op::NEEDS_LIVE) return seg_live<KT>(c, seg);
-    else return true;
+__device__ __forceinline__ bool op_stage(const Ctx &c, const Op &op, int seg, double *sh) {
+    __shared__ int s_need;
+    if (threadIdx.x < 32) {
+        const int j = threadIdx.x;
+        int need = 1;
+        if constexpr (LiveOnStep<Op>::value)
+            need = __any_sync(NVD_FULLMASK, __ldcg(c.alpha + (int64_t)seg * KT + j % KT) != 0.0);
+        else if constexpr (Op::NEEDS_LIVE)
+            need = __any_sync(NVD_FULLMASK, __ldcg(c.active + (int64_t)seg * KT + j % KT) != 0);
+        if (j < KT) op.stage(c, (int64_t)seg * KT + j, j, KT, sh);
+        if (j == 0) s_need = need;
+    }
+    __syncthreads();
+    return s_need != 0;
 }
 
 // Generic streaming pass over rows [i0, i1) of one segment.  Op provides ND,
-// NEEDS_LIVE (see op_live), a register type R, setup(c, seg, col0), load(c, i,
-// col0, R&) and apply(c, i, col0, R&, dot) with per-thread partial sums of type
+// NEEDS_LIVE, stage(c, i, j, KT, sh) (column j's scalars, state index i, into shared memory;
+// see op_stage), a register type R, setup(c, seg, col0, sh), load(c, i, col0, R&) and apply(c, i, col0, R&, dot) with per-thread partial sums of type
 // Op::D (see DotOf).  Each thread handles U lane-vectors per trip with all U loads
 // issued before the first use.
 template <class TV, int KT, class Op, int U = 4>
@@ -52,8 +60,8 @@ __device__ void vec_block(const Ctx &c, Op op, int64_t b, char *smem) {
     for (int d = 0; d < (ND > 0 ? ND : 1); ++d)
 #pragma unroll
         for (int v = 0; v < VEC; ++v) dot_zero(dot[d][v]);
-    if (op_live<KT, Op>(c, seg)) {
-        op.setup(c, seg, col0);
+    if (op_stage<KT, Op>(c, op, seg, tot)) {
+        op.setup(c, seg, col0, tot);
         const int64_t t1 = blk.i1 * CG;
         for (int64_t t = blk.i0 * CG + threadIdx.x; t < t1; t += (int64_t)NT * U) {
             typename Op::R regs[U];
@@ -92,7 +100,8 @@ struct OpFormDelta {
     const TX *X, *Y;
     int64_t base, ld;
     int kc, idx;
-    __device__ void setup(const Ctx &c, int seg, int) {
+    __device__ __forceinline__ void stage(const Ctx &, int64_t, int, int, double *) const {}
+    __device__ void setup(const Ctx &c, int seg, int, const double *) {
         const Owner &o = owner_of(c, seg);
         X = reinterpret_cast<const TX *>(o.x);
         Y = reinterpret_cast<const TX *>(o.y);
@@ -140,9 +149,12 @@ struct OpInit {
     bool zero_x = true;   // false: keep x (warm start)
     FinInit fin;
     double mu[VEC];
-    __device__ void setup(const Ctx &c, int seg, int col0) {
+    __device__ __forceinline__ void stage(const Ctx &c, int64_t i, int j, int, double *sh) const {
+        sh[j] = __ldcg(c.mean + i);
+    }
+    __device__ void setup(const Ctx &, int, int col0, const double *sh) {
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) mu[v] = __ldcg(c.mean + (int64_t)seg * KT + col0 + v);
+        for (int v = 0; v < VEC; ++v) mu[v] = sh[col0 + v];
     }
     __device__ __forceinline__ void load(const Ctx &c, int64_t i, int col0, R &q) const {
         ldv<LD, double, VEC>(src + i * KT + col0, q.s);
@@ -180,7 +192,8 @@ struct OpLoadX {
     FinNone fin;
     int64_t base, ld;
     int kc;
-    __device__ void setup(const Ctx &c, int seg, int) {
+    __device__ __forceinline__ void stage(const Ctx &, int64_t, int, int, double *) const {}
+    __device__ void setup(const Ctx &c, int seg, int, const double *) {
         const Owner &o = owner_of(c, seg);
         base = o.base;
         ld = o.ld;
@@ -215,9 +228,12 @@ struct OpUpdate {
     TV *u = nullptr;
     FinBeta fin;
     TV al[VEC];
-    __device__ void setup(const Ctx &c, int seg, int col0) {
+    __device__ __forceinline__ void stage(const Ctx &c, int64_t i, int j, int, double *sh) const {
+        sh[j] = __ldcg(c.alpha + i);
+    }
+    __device__ void setup(const Ctx &, int, int col0, const double *sh) {
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) al[v] = (TV)__ldcg(c.alpha + (int64_t)seg * KT + col0 + v);
+        for (int v = 0; v < VEC; ++v) al[v] = (TV)sh[col0 + v];
     }
     __device__ __forceinline__ void load(const Ctx &c, int64_t i, int col0, R &g) const {
         const int64_t o = i * KT + col0;
@@ -263,9 +279,12 @@ struct OpResid {
     const TV *q;
     FinBeta fin;
     TV al[VEC];
-    __device__ void setup(const Ctx &c, int seg, int col0) {
+    __device__ __forceinline__ void stage(const Ctx &c, int64_t i, int j, int, double *sh) const {
+        sh[j] = __ldcg(c.alpha + i);
+    }
+    __device__ void setup(const Ctx &, int, int col0, const double *sh) {
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) al[v] = (TV)__ldcg(c.alpha + (int64_t)seg * KT + col0 + v);
+        for (int v = 0; v < VEC; ++v) al[v] = (TV)sh[col0 + v];
     }
     __device__ __forceinline__ void load(const Ctx &c, int64_t i, int col0, R &g) const {
         const int64_t o = i * KT + col0;
@@ -303,13 +322,17 @@ struct OpStepDir {
     FinNone fin;
     TV al[VEC], be[VEC];
     bool act[VEC];
-    __device__ void setup(const Ctx &c, int seg, int col0) {
+    __device__ __forceinline__ void stage(const Ctx &c, int64_t i, int j, int, double *sh) const {
+        sh[j] = __ldcg(c.alpha + i);
+        sh[KT + j] = __ldcg(c.beta + i);
+        sh[2 * KT + j] = __ldcg(c.active + i) != 0 ? 1.0 : 0.0;
+    }
+    __device__ void setup(const Ctx &, int, int col0, const double *sh) {
 #pragma unroll
         for (int v = 0; v < VEC; ++v) {
-            const int64_t i = (int64_t)seg * KT + col0 + v;
-            al[v] = (TV)__ldcg(c.alpha + i);
-            be[v] = (TV)__ldcg(c.beta + i);
-            act[v] = __ldcg(c.active + i) != 0;
+            al[v] = (TV)sh[col0 + v];
+            be[v] = (TV)sh[KT + col0 + v];
+            act[v] = __double2hiint(sh[2 * KT + col0 + v]) != 0;
         }
     }
     __device__ __forceinline__ void load(const Ctx &c, int64_t i, int col0, R &g) const {
@@ -341,7 +364,8 @@ struct OpFinal {
     const TV *x;
     const double *delta;
     FinFinal fin;
-    __device__ void setup(const Ctx &, int, int) {}
+    __device__ __forceinline__ void stage(const Ctx &, int64_t, int, int, double *) const {}
+    __device__ void setup(const Ctx &, int, int, const double *) {}
     __device__ __forceinline__ void load(const Ctx &, int64_t i, int col0, R &g) const {
         const int64_t o = i * KT + col0;
         ldv<LD, TV, VEC>(x + o, g.x);
@@ -370,14 +394,17 @@ struct OpZout {
     int64_t base, ld;
     int kc;
     double mu[VEC];
-    __device__ void setup(const Ctx &c, int seg, int col0) {
+    __device__ __forceinline__ void stage(const Ctx &, int64_t i, int j, int, double *sh) const {
+        sh[j] = __ldcg(meanv + i);
+    }
+    __device__ void setup(const Ctx &c, int seg, int col0, const double *sh) {
         const Owner &o = owner_of(c, seg);
         Z = reinterpret_cast<TZ *>(o.z);
         base = o.base;
         ld = o.ld;
         kc = o.kc;
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) mu[v] = __ldcg(meanv + (int64_t)seg * KT + col0 + v);
+        for (int v = 0; v < VEC; ++v) mu[v] = sh[col0 + v];
     }
     __device__ __forceinline__ void load(const Ctx &, int64_t i, int col0, R &g) const {
         ldv<LD, TS, VEC>(src + i * KT + col0, g.s);
@@ -403,7 +430,8 @@ struct OpAccum {
     const TV *x;
     double *z;
     FinNone fin;
-    __device__ void setup(const Ctx &, int, int) {}
+    __device__ __forceinline__ void stage(const Ctx &, int64_t, int, int, double *) const {}
+    __device__ void setup(const Ctx &, int, int, const double *) {}
     __device__ __forceinline__ void load(const Ctx &, int64_t i, int col0, R &g) const {
         const int64_t o = i * KT + col0;
         ldv<LD, TV, VEC>(x + o, g.x);
