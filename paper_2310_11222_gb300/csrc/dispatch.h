@@ -38,7 +38,9 @@ int ge_distance_internal(nvd_graph_t g, int32_t k, const void *x, const void *y,
 int elim_distance(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_t xdt,
                   const nvd_solve_opts *opts, double *d2_out, void *z_out, nvd_solve_stats *stats,
                   cudaStream_t s, bool idx = false);
-// y = L x for one contiguous column (internal order), dtype = F32 or F64.
-int run_apply(nvd_graph_s *g, const Ctx &c, const void *x, void *y, int dtype, cudaStream_t s);
+// y = L x for k vectors ld elements apart (internal order), dtype = F32 or F64.  split: the
+// plan has rows split over several blocks.
+int run_apply(nvd_graph_s *g, const Ctx &c, int k, const void *x, void *y, int64_t ld, bool split, int dtype,
+              cudaStream_t s);
 
 }  // namespace nvd

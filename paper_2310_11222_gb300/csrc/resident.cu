@@ -630,14 +630,14 @@ int launch(const ResidentPlan *pl, const RsArgs &a, cudaStream_t s) {
 }  // namespace
 
 // Fitted to measured runs: three meetings and two sums 16 us; the FP64 instructions, 15% of the
-// entries and 20% in all lost to padding and imbalance; one column is bound by its gathers, 1.3
+// entries and 35% in all lost to padding and imbalance (20% on ER graphs, 45% on BA); one column is bound by its gathers, 1.3
 // clocks each, and from about 150,000 rows on by the loads L1 can keep in flight beside the
 // vectors in shared memory.
 double resident_iter_us(int64_t n, int64_t nnz, int KT) {
     const double mhz = 2000.0, sms = 152.0;
     if (KT == 1)
         return 16.0 + 9.0 * (double)n / (2.0 * sms) / mhz + 1.3 * (double)nnz / sms / mhz * (n > 150000 ? 1.8 : 1.0);
-    return 16.0 + 1.2 * KT * (1.15 * (double)nnz + 9.0 * (double)n) / (2.0 * sms) / mhz;
+    return 16.0 + 1.35 * KT * (1.15 * (double)nnz + 9.0 * (double)n) / (2.0 * sms) / mhz;
 }
 
 int resident_plan_for(nvd_graph_s *g, int KT, ResidentPlan **out) {

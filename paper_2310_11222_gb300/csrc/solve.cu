@@ -778,16 +778,18 @@ int apply_impl(nvd_graph_t g, int32_t k, const void *x, void *y, int32_t dtype, 
         yout = g->wsp("apply_y", g->n * sz, &st);
         if (st) return st;
     }
-    NVD_TRY_CUDA(cudaMemsetAsync(y, 0, (size_t)k * g->n * sz, s));
-    for (int32_t j = 0; j < k; ++j) {
-        const char *xj = (const char *)x + (size_t)j * g->n * sz;
-        char *yj = (char *)y + (size_t)j * g->n * sz;
-        if (!g->perm.p) {
-            NVD_TRY(run_apply(g, c, xj, yj, dtype, s));
-        } else {
+    // isolated nodes belong to no block
+    if (g->n_singleton > 0) NVD_TRY_CUDA(cudaMemsetAsync(y, 0, (size_t)k * g->n * sz, s));
+    const bool split = pl->n_chunks > 0;
+    if (!g->perm.p) {
+        NVD_TRY(run_apply(g, c, k, x, y, g->n, split, dtype, s));
+    } else {
+        for (int32_t j = 0; j < k; ++j) {
+            const char *xj = (const char *)x + (size_t)j * g->n * sz;
+            char *yj = (char *)y + (size_t)j * g->n * sz;
             NVD_TRY(permute_vector(xj, xin, g->perm.as<int32_t>(), g->n, dtype, true, s));
-            NVD_TRY_CUDA(cudaMemsetAsync(yout, 0, g->n * sz, s));
-            NVD_TRY(run_apply(g, c, xin, yout, dtype, s));
+            if (g->n_singleton > 0) NVD_TRY_CUDA(cudaMemsetAsync(yout, 0, g->n * sz, s));
+            NVD_TRY(run_apply(g, c, 1, xin, yout, g->n, split, dtype, s));
             NVD_TRY(permute_vector(yout, yj, g->perm.as<int32_t>(), g->n, dtype, false, s));
         }
     }

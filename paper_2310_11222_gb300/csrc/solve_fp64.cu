@@ -1,4 +1,6 @@
 // FP64-mode tile solver instantiations (KT in {1,4,8,16,32} x weight type x input type).
+#include <algorithm>
+
 #include "dispatch.h"
 #include "solver.cuh"
 
@@ -44,16 +46,36 @@ int run_collect(const Ctx &c, int KT, ColResult *res, double *d2dev, int64_t d2_
     return NVD_OK;
 }
 
-int run_apply(nvd_graph_s *g, const Ctx &c, const void *x, void *y, int dtype, cudaStream_t s) {
-    dev::EpiApply epi;
-    if (dtype == NVD_F64) {
-        const double bytes = spmm_bytes(g, 1, 8, g->wdtype == NVD_F64 ? 8 : 4, 8);
-        if (g->wdtype == NVD_F64)
-            return launch_spmm<double, double, double, 1>(c, epi, (const double *)x, (double *)y, s, bytes);
-        return launch_spmm<double, float, double, 1>(c, epi, (const double *)x, (double *)y, s, bytes);
+namespace {
+// k vectors ld elements apart.
+template <class TV, class TW, class TA>
+int apply_vectors(nvd_graph_s *g, const Ctx &c, int k, const TV *x, TV *y, int64_t ld, bool split, cudaStream_t s) {
+    if (c.n_sblk == 0) return NVD_OK;
+    if (!split && !prof_enabled()) {
+        for (int j = 0; j < k; j += 65535) {
+            const dim3 grid((unsigned)c.n_sblk, (unsigned)std::min(k - j, 65535));
+            k_apply<TV, TW, TA><<<grid, NT, 0, s>>>(c, x + j * ld, y + j * ld, ld);
+            note_launch();
+            NVD_TRY_CUDA(cudaGetLastError());
+        }
+        return NVD_OK;
     }
-    const double bytes = spmm_bytes(g, 1, 4, 4, 4);
-    return launch_spmm<float, float, float, 1>(c, epi, (const float *)x, (float *)y, s, bytes);
+    const dev::EpiApply epi;
+    const double bytes = spmm_bytes(g, 1, sizeof(TV), sizeof(TW), sizeof(TA));
+    for (int j = 0; j < k; ++j)
+        NVD_TRY((launch_spmm<TV, TW, TA, 1>(c, epi, x + j * ld, y + j * ld, s, bytes)));
+    return NVD_OK;
+}
+}  // namespace
+
+int run_apply(nvd_graph_s *g, const Ctx &c, int k, const void *x, void *y, int64_t ld, bool split, int dtype,
+              cudaStream_t s) {
+    if (dtype == NVD_F64) {
+        if (g->wdtype == NVD_F64)
+            return apply_vectors<double, double, double>(g, c, k, (const double *)x, (double *)y, ld, split, s);
+        return apply_vectors<double, float, double>(g, c, k, (const double *)x, (double *)y, ld, split, s);
+    }
+    return apply_vectors<float, float, float>(g, c, k, (const float *)x, (float *)y, ld, split, s);
 }
 
 }  // namespace nvd

@@ -60,6 +60,17 @@ __global__ void __launch_bounds__(NT, KT == 1 ? NVD_SPMV1_MINB : NVD_SPMM_MINB) 
     dev::spmm_block<dev::LdRO, TV, TW, TA, KT, Epi>(c, epi, src, dst, blockIdx.x, smem);
 }
 
+// y = L x of one vector per grid row (blockIdx.y), vectors ld elements apart, in one launch: six
+// launches one after the other on 300,000 rows took 18 us each, 6 of them FP64 work.  Not for
+// plans with rows split over blocks, whose partial sums have one place per launch.
+template <class TV, class TW, class TA>
+__global__ void __launch_bounds__(NT, NVD_SPMV1_MINB) k_apply(Ctx c, const TV *src, TV *dst, int64_t ld) {
+    __shared__ __align__(16) char smem[dev::SpCfg<TV, TA, 1>::SMEM];
+    const dev::EpiApply epi;
+    dev::spmm_block<dev::LdRO, TV, TW, TA, 1, dev::EpiApply>(c, epi, src + blockIdx.y * ld, dst + blockIdx.y * ld,
+                                                             blockIdx.x, smem);
+}
+
 // The multi-column SpMM over a stream plan (stream.cuh).  Register engine: three CTAs
 // per SM (85 registers a thread).  TMA engine (rows of 64 or 128 bytes): two CTAs per
 // SM, each with NWARP rings of TMA_SLOTS 512-byte steps in dynamic shared memory.
