@@ -24,8 +24,9 @@ constexpr int sp_row_max(int KT, int szv) { return KT == 1 ? 128 : 32768 / (KT *
 constexpr int sp_long_max(int KT) { return KT == 1 ? 8192 : 0; }
 constexpr int sp_chunk(int KT, int szv) { return KT == 1 ? 4096 : 32768 / (KT * szv); }
 // Rows (first to last) one single-column light SpMV block may span: its row sums
-// are staged in shared memory by row so the row epilogue runs in row order.
-constexpr int sp_span_max() { return 1024; }
+// are staged in shared memory by row so the row epilogue runs in row order.  (With 1,024, 10^6
+// rows made 977 blocks, one wave and a 0.6 of another: 17.0 ms per 8 solves against 16.5.)
+constexpr int sp_span_max() { return 2048; }
 // d^2 stop: the gap estimate takes the largest of the last d2_window ratios of
 // consecutive d^2 increments (window and safety factor chosen on recorded CG
 // traces of ER, BA, WS and SBM graphs of mean degree 2..32, paths and cycles).
@@ -44,8 +45,9 @@ constexpr int sp_slice_rows(int KT, int szv) { return 32 / sp_lanes_per_row(KT, 
 // results.
 constexpr int sp_group_max(int KT, int szv) { return KT > 1 && szv == 8 ? 32 : INT32_MAX; }
 // doubles of reduction scratch per CTA: every thread's partial of up to 4 sums (one column,
-// added by one warp per sum), or of the 4 columns a thread holds of one sum
-constexpr int red_doubles(int) { return 4 * NT; }
+// added by one warp per sum; before that the block's row sums), or of the 4 columns a thread
+// holds of one sum
+constexpr int red_doubles(int KT) { return KT == 1 ? sp_span_max() : 4 * NT; }
 constexpr int vec_smem_bytes(int KT) { return (red_doubles(KT) + 4 * KT) * 8; }
 // Stream plans of multi-column tiles (stream.cuh): light rows of at most
 // 256 / H entries (longer slices would unbalance the warps of a block), heavy rows cut

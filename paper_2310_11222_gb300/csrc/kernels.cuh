@@ -177,7 +177,7 @@ __device__ __forceinline__ double f2d(float f) {
     return m == 0 ? __hiloint2double((int)b, 0) : (double)f;
 }
 __device__ __forceinline__ double dot_get(const DFloat &d) { return f2d(d.hi) + f2d(d.lo); }
-// A stored weight in the accumulator type.
+// A weight (or sum) in the accumulator type.
 template <class TA, class TW>
 __device__ __forceinline__ TA weight_as(TW w) {
     if constexpr (sizeof(TA) == 8 && sizeof(TW) == 4) return f2d(w);
@@ -877,7 +877,7 @@ __device__ __forceinline__ void spmm_chunk(const Ctx &c, const Epi &epi, int seg
             for (int v = 0; v < VEC; ++v) acc[v] += __shfl_xor_sync(NVD_FULLMASK, acc[v], off);
         if (gi == 0) {
 #pragma unroll
-            for (int v = 0; v < VEC; ++v) red[KT + warp * KT + col0 + v] = (double)acc[v];
+            for (int v = 0; v < VEC; ++v) red[KT + warp * KT + col0 + v] = weight_as<double>(acc[v]);
         }
         __syncthreads();
         if (threadIdx.x < KT) {
@@ -1319,9 +1319,14 @@ __device__ void spmm_block(const Ctx &c, const Epi &epi, const TV *__restrict__ 
         }
     }
     if constexpr (ND > 0) {
-        double dd[ND][VEC];
-        dot_to_double(dot, dd);
-        block_reduce_cols<ND, KT, VEC>(dd, red, tot);
+        if (blk.pad == 0) {
+            double dd[ND][VEC];
+            dot_to_double(dot, dd);
+            block_reduce_cols<ND, KT, VEC>(dd, red, tot);
+        } else {            // split rows' products go to their own slots
+            if (threadIdx.x < ND * KT) tot[threadIdx.x] = 0.0;
+            __syncthreads();
+        }
         const int64_t s0 = c.seg_sblk_off[seg];
         const int32_t cnt = c.seg_sblk_off[seg + 1] - (int32_t)s0;
         const int64_t h0 = c.n_sblk + c.seg_heavy_off[seg];
