@@ -14,10 +14,10 @@ int cluster_estimate(nvd_graph_s *g, int64_t cols, int *cs, double *us);
 int cluster_plan_get(nvd_graph_s *g, int cs, ClusterPlan **out);
 // Estimated microseconds of one iteration of the host-driven loop on `tiles` tiles of kt FP64
 // columns, fitted to runs from 3 * 10^4 to 10^6 rows: three launches and their block reductions,
-// and 1.4 times the FP64 instructions (a multiply-add per entry and 10 operations per row, at 2
+// and 1.35 times the FP64 instructions (a multiply-add per entry and 10 operations per row, at 2
 // lanes per SM and clock).
 inline double tiles_iter_us(int64_t n, int64_t nnz, int kt, int tiles) {
-    return tiles * (32.0 + 2.0 * kt + 1.4 * kt * ((double)nnz + 10.0 * (double)n) / 6.3e5);
+    return tiles * (32.0 + 0.6 * kt + 1.35 * kt * ((double)nnz + 10.0 * (double)n) / 6.3e5);
 }
 
 // Solve K columns for every owner (owners_dev: device table of n_owner, or NULL: own0);

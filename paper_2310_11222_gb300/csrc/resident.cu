@@ -10,14 +10,14 @@
 // itself, in a fixed order: no second meeting, and every CTA takes the same scalars.
 //
 // Against the three launches of the host-driven loop this saves their ramps, tails and block
-// reductions and the vectors' trips to L2.  Microseconds per iteration (before: host-driven):
-// ER graph of 30,000 nodes, mean degree 10: 1 / 4 / 8 / 16 columns 17 / 20 / 25 / 35 (34 / 45 /
-// 58 / 89); of 100,000 nodes 1 / 4 / 8 columns 21 / 29 / 43 (41 / 56 / 80); ring of 200,000, one
-// column 20 (36).  One column of 10^6 nodes is left to the host-driven loop (116 against 95):
-// with 174 KB of vectors in shared memory L1 holds too few of the gathers in flight.  What
-// bounds it now: the FP64 pipe from 8 columns on (100,000 nodes: row sums 33,600 of 82,900
-// clocks, vector passes 20,000); below, the two sums (10,000 clocks each, 4,000 of them the
-// meeting) and the chain of dependent loads in the row sums.
+// reductions and the vectors' trips to L2.  Microseconds per iteration (host-driven): ER graph
+// of 30,000 nodes, mean degree 10: 1 / 4 / 8 / 16 columns 15 / 18 / 23 / 30 (32 / 41 / 45 / 57);
+// of 100,000 nodes 1 / 4 / 8 columns 19 / 27 / 40 (39 / 50 / 67); BA graph of 300,000, one column
+// 36 (66).  One column of 10^6 nodes is left to the host-driven loop (116 against 89): with
+// 174 KB of vectors in shared memory L1 holds too few of the gathers in flight.  What bounds it:
+// the FP64 pipe from 8 columns on (100,000 nodes: row sums 33,600 of 80,000 clocks, vector
+// passes 17,000); below, the two sums (9,000 clocks each, 4,000 of them the meeting) and the
+// chain of dependent loads in the row sums.
 //
 // The grid barrier's wait is bounded (2 s): a CTA that gives up records NVD_ERR_TIMEOUT in
 // the error word and leaves; all CTAs are co-resident (cooperative launch), so this can
@@ -96,13 +96,16 @@ __device__ __forceinline__ uint64_t timer_ns() {
 }
 
 // All CTAs; every thread's writes before it are seen after it.  target: arrivals so far.
-__device__ __forceinline__ bool grid_meet(const RsArgs &a, RsState &st, unsigned &target) {
+// `meanwhile` runs between this CTA's arrival and its wait (work no other CTA asks for).
+template <class W>
+__device__ __forceinline__ bool grid_meet(const RsArgs &a, RsState &st, unsigned &target, W meanwhile) {
     target += gridDim.x;
     __syncthreads();
+    // release and acquire at GPU scope order the whole CTA's writes and reads through the
+    // block barriers around them
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
+    meanwhile();
     if (threadIdx.x == 0) {
-        // release and acquire at GPU scope order the whole CTA's writes and reads through the
-        // block barriers around them
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
         unsigned seen;
         const uint64_t t0 = timer_ns();
         for (unsigned spin = 1;; ++spin) {
@@ -143,9 +146,9 @@ __device__ __forceinline__ double sum256(double *red, int id, int t, double v) {
 // Column sums over the grid of every thread's v0 (and v1), the thread's column being
 // threadIdx.x % KT; fin(j, s0, s1) runs in thread j < KT of every CTA, with the same values.
 // Returns false if a wait gave up.  `red` holds NV * RS_NT doubles.
-template <int KT, int NV, class F>
+template <int KT, int NV, class F, class W>
 __device__ __forceinline__ bool grid_sum(const RsArgs &a, RsState &st, double *red, unsigned &target, int &par, double v0,
-                                         double v1, F fin) {
+                                         double v1, F fin, W meanwhile) {
     constexpr int S = NV * KT;
     const int t = threadIdx.x;
     double *part = a.part + (int64_t)par * gridDim.x * 2 * KT;
@@ -160,7 +163,7 @@ __device__ __forceinline__ bool grid_sum(const RsArgs &a, RsState &st, double *r
         const double s = sum256<KT>(rv, v, tt, m);
         if (tt < KT) part[(int64_t)blockIdx.x * S + v * KT + tt] = s;
     }
-    if (!grid_meet(a, st, target)) return false;
+    if (!grid_meet(a, st, target, meanwhile)) return false;
     if (t < 256) {
         // all CTAs' sums: thread t adds sum t % S of CTAs t / S, t / S + 256 / S, ...
         double s = 0.0;
@@ -203,6 +206,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
     const double *__restrict__ wv = a.w + ct.e0;
     unsigned target = 0;
     int par = 0;
+    auto nothing = []() {};
 
     auto delta_at = [&](int s) -> double {
         if (j >= a.own.kc) return 0.0;
@@ -233,7 +237,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
         s0 += d;
     }
     __syncthreads();
-    if (!(grid_sum<KT, 1>(a, st, red, target, par, s0, 0.0, [&](int c, double s, double) { st.mean[c] = s / (double)a.n; })))
+    if (!(grid_sum<KT, 1>(a, st, red, target, par, s0, 0.0, [&](int c, double s, double) { st.mean[c] = s / (double)a.n; }, nothing)))
         return;
     s0 = 0.0;
     for (int e = tid; e < ne; e += RS_NT) {
@@ -257,7 +261,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
             const unsigned all = KT == 32 ? 0xffffffffu : (1u << KT) - 1u;
             const unsigned any = __ballot_sync(all, act);
             if (c == 0) st.go = any != 0;
-        })))
+        }, nothing)))
         return;
     while (st.go) {
         // row sums of W p: warps take the CTA's items, longest first
@@ -347,13 +351,12 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
                     st.alpha[c] = 0.0;
                     st.status[c] = NVD_ERR_NUMERIC;
                 }
-            })))
+            }, nothing)))
             return;
-        // x += alpha p, r -= alpha q, u = D^-1 r (kept in q); r^T u and |r|^2
+        // r -= alpha q, u = D^-1 r (kept in q); r^T u and |r|^2; x += alpha p while the CTAs meet
         const double al = st.alpha[j];
         s0 = s1 = 0.0;
         for (int e = tid; e < ne; e += RS_NT) {
-            x[e] = fma(al, p[e], x[e]);
             const double rv = fma(-al, q[e], r[e]);
             const double u = __ldg(dinv + e / KT) * rv;
             r[e] = rv;
@@ -399,6 +402,9 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
                 const unsigned all = KT == 32 ? 0xffffffffu : (1u << KT) - 1u;
                 const unsigned any = __ballot_sync(all, act);
                 if (c == 0) st.go = any != 0;
+            },
+            [&]() {
+                for (int e = tid; e < ne; e += RS_NT) x[e] = fma(al, p[e], x[e]);
             })))
             return;
         if (!st.go) break;
@@ -410,7 +416,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
                 pg[e] = v;
             }
         }
-        if (!grid_meet(a, st, target)) return;
+        if (!grid_meet(a, st, target, nothing)) return;
     }
     // d^2 = delta^T x (delta projected), the mean of x, z = x - mean
     s0 = s1 = 0.0;
@@ -422,7 +428,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
     if (!(grid_sum<KT, 2>(a, st, red, target, par, s0, s1, [&](int c, double sx, double dx) {
             st.beta[c] = sx / (double)a.n;
             st.d2[c] = dx;
-        })))
+        }, nothing)))
         return;
     if (a.write_z && j < a.own.kc) {
         const double mu = st.beta[j];
