@@ -557,8 +557,9 @@ ClLimits cl_limits(int64_t rows_per_cta) {
 int64_t cl_spc_estimate(int64_t n, int cs) { return ((n + cs - 1) / cs + 31) / 32 * 32 + 64; }
 
 int fill_cluster_plan(nvd_graph_s *g, ClusterPlan *pl, cudaStream_t s) {
-    return fill_onchip(g, pl->n_tasks, 32, pl->tasks, pl->slot_of, pl->col, pl->w, pl->n_slots, pl->slot_row, pl->deg,
-                       pl->dinv, s);
+    return fill_onchip(g, pl->n_tasks, 32, pl->tasks.as<FillTask>(), pl->slot_of.as<int32_t>(), pl->col.as<int32_t>(),
+                       pl->w.as<double>(), pl->n_slots, pl->slot_row.as<int32_t>(), pl->deg.as<double>(),
+                       pl->dinv.as<double>(), s);
 }
 
 // CTAs per cluster of a component of n rows when the largest uses cs_max: one up to 512 rows

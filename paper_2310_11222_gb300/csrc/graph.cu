@@ -699,11 +699,16 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
     std::vector<int32_t> seg_sblk_off(nseg + 1, 0);
     std::vector<int64_t> sl_base(1, 0);
     std::vector<int32_t> sl_row;
-    std::vector<int64_t> rows, lens;
+    std::vector<int64_t> rows, lens, ord, place;
     auto emit_block = [&](int s) {
-        std::vector<int64_t> ord(rows.size());
-        for (size_t q = 0; q < ord.size(); ++q) ord[q] = (int64_t)q;
-        std::stable_sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) { return lens[x] > lens[y]; });
+        // longest first, ties by row: a counting sort over the lengths
+        int64_t lmax = 0;
+        for (int64_t d : lens) lmax = std::max(lmax, d);
+        place.assign(lmax + 2, 0);
+        for (int64_t d : lens) ++place[lmax - d + 1];
+        for (int64_t d = 0; d <= lmax; ++d) place[d + 1] += place[d];
+        ord.resize(rows.size());
+        for (size_t q = 0; q < ord.size(); ++q) ord[place[lmax - lens[q]]++] = (int64_t)q;
         const int64_t first = (int64_t)sl_base.size() - 1;
         size_t q0 = 0;
         for (; q0 < ord.size() && lens[ord[q0]] > GMAX; ++q0) {   // a row over all lane groups

@@ -70,21 +70,19 @@ static __global__ void k_fill_deg(int64_t n, const int32_t *__restrict__ row, co
 }
 
 // Fill a plan's entries and degrees from the graph (at creation and for new weights).
-inline int fill_onchip(const nvd_graph_s *g, int64_t n_tasks, int H, const DevBuf &tasks, const DevBuf &slot_of,
-                       const DevBuf &col, const DevBuf &w, int64_t n_slots, const DevBuf &slot_row, const DevBuf &deg,
-                       const DevBuf &dinv, cudaStream_t s) {
+inline int fill_onchip(const nvd_graph_s *g, int64_t n_tasks, int H, const FillTask *tasks, const int32_t *slot_of,
+                       int32_t *col, double *w, int64_t n_slots, const int32_t *slot_row, double *deg, double *dinv,
+                       cudaStream_t s) {
     if (n_slots == 0) return NVD_OK;
     const int64_t warps = n_tasks > n_slots ? n_tasks : n_slots;
     const int64_t cap = (int64_t)g->num_sms * 16, want = (warps + 7) / 8;
     const int grid = (int)(want < cap ? want : cap);
     auto go = [&](auto *wg) {
-        k_fill<<<grid, 256, 0, s>>>(n_tasks, H, tasks.as<FillTask>(), slot_of.as<int32_t>(), g->colidx.as<int32_t>(),
-                                    wg, col.as<int32_t>(), w.as<double>());
+        k_fill<<<grid, 256, 0, s>>>(n_tasks, H, tasks, slot_of, g->colidx.as<int32_t>(), wg, col, w);
     };
     if (g->wdtype == NVD_F64) go(g->w.as<double>());
     else go(g->w.as<float>());
-    k_fill_deg<<<grid, 256, 0, s>>>(n_slots, slot_row.as<int32_t>(), g->deg64.as<double>(), g->dinv64.as<double>(),
-                                    deg.as<double>(), dinv.as<double>());
+    k_fill_deg<<<grid, 256, 0, s>>>(n_slots, slot_row, g->deg64.as<double>(), g->dinv64.as<double>(), deg, dinv);
     NVD_TRY_CUDA(cudaGetLastError());
     return NVD_OK;
 }

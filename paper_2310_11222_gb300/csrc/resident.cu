@@ -451,8 +451,16 @@ struct ResidentPlan {
     bool x_global = false, fits = false;
     size_t smem = 0;
     int64_t n_slots = 0;
-    DevBuf ctas, items, splits, col, w, node, deg, dinv;
-    DevBuf tasks, slot_row, slot_of;   // what the weight updates need
+    // two allocations and one copy: with one each, a new graph's first call took 10 ms instead
+    // of 4 at 100,000 nodes (the rest of that was a comparison sort)
+    DevBuf meta, data;
+    RsCta *ctas = nullptr;
+    Item *items = nullptr;
+    RsSplit *splits = nullptr;
+    int32_t *node = nullptr, *col = nullptr;
+    double *w = nullptr, *deg = nullptr, *dinv = nullptr;
+    FillTask *tasks = nullptr;         // with slot_row, slot_of: what the weight updates need
+    int32_t *slot_row = nullptr, *slot_of = nullptr;
     int64_t n_tasks = 0;
 };
 
@@ -470,10 +478,7 @@ int64_t resident_state_bytes(const ResidentState *c) {
     int64_t b = 0;
     if (c)
         for (auto &kv : c->plans)
-            for (const DevBuf *d : {&kv.second->ctas, &kv.second->items, &kv.second->splits, &kv.second->col,
-                                    &kv.second->w, &kv.second->node, &kv.second->deg, &kv.second->dinv,
-                                    &kv.second->tasks, &kv.second->slot_row, &kv.second->slot_of})
-                b += (int64_t)d->bytes;
+            b += (int64_t)(kv.second->meta.bytes + kv.second->data.bytes);
     return b;
 }
 
@@ -507,6 +512,9 @@ int build_resident_plan(nvd_graph_s *g, int KT, ResidentPlan **out) {
     std::vector<FillTask> tasks;
     std::vector<int32_t> node, slot_row, slot_of(g->n, 0);
     std::vector<int64_t> ord;
+    tasks.reserve(n + n / 16);
+    node.reserve(n);
+    slot_row.reserve(n);
     // Rows of more than 32 entries are dealt to the CTAs back and forth, longest first (hubs
     // often come together in the node order, and the CTAs meet after the row sums and after the
     // vector passes: each needs its share of both; by running work alone the CTAs with the hubs
@@ -529,13 +537,24 @@ int build_resident_plan(nvd_graph_s *g, int KT, ResidentPlan **out) {
             const int64_t at = round * P + ((round & 1) ? P - 1 - c : c);
             if (at < (int64_t)wide.size()) ord.push_back(wide[at]);
         }
+        // the light rows of its range by length, longest first (at most 32 entries: counting sort)
         const double until = total * (c + 1) / P;
+        const int64_t r0 = r;
+        int64_t at[34] = {0};
         for (; r < a + n; ++r) {
-            if (len_of(r) > 32) continue;
-            const double work = (double)len_of(r) + 9.0;
+            const int64_t d = len_of(r);
+            if (d > 32) continue;
+            const double work = (double)d + 9.0;
             if (c < P - 1 && done + 0.5 * work > until) break;
             done += work;
-            ord.push_back(r);
+            ++at[33 - d];
+        }
+        for (int d = 1; d < 34; ++d) at[d] += at[d - 1];
+        const int64_t nwide = (int64_t)ord.size();
+        ord.resize(nwide + at[33]);
+        for (int64_t i = r0; i < r; ++i) {
+            const int64_t d = len_of(i);
+            if (d <= 32) ord[nwide + at[32 - d]++] = i;
         }
         const int64_t nr = (int64_t)ord.size();
         RsCta &ct = ctas[c];
@@ -545,7 +564,6 @@ int build_resident_plan(nvd_graph_s *g, int KT, ResidentPlan **out) {
         ct.split0 = (int64_t)splits.size();
         ct.e0 = ne;
         ct.nslot = (int32_t)nr;
-        std::stable_sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) { return len_of(x) > len_of(y); });
         for (int64_t i = 0; i < nr; ++i) {
             const int64_t row = ord[i];
             slot_of[row] = (int32_t)(ct.slot0 + i);
@@ -591,22 +609,36 @@ int build_resident_plan(nvd_graph_s *g, int KT, ResidentPlan **out) {
     pl->smem = rs_smem(max_rows, max_extra, KT, pl->x_global);
     pl->fits = pl->smem <= RS_SMEM_MAX;
     if (pl->fits) {
-        auto up = [&](DevBuf &d, const void *h, size_t bytes) -> int {
-            NVD_TRY(d.alloc(std::max<size_t>(bytes, 16)));
-            if (bytes) NVD_TRY_CUDA(cudaMemcpy(d.p, h, bytes, cudaMemcpyHostToDevice));
-            return NVD_OK;
+        std::vector<char> host;
+        size_t off[7];
+        auto add = [&](int i, const void *h, size_t bytes) {
+            off[i] = host.size();
+            host.resize(off[i] + (bytes + 255) / 256 * 256);
+            if (bytes) memcpy(host.data() + off[i], h, bytes);
         };
-        NVD_TRY(up(pl->ctas, ctas.data(), ctas.size() * sizeof(RsCta)));
-        NVD_TRY(up(pl->items, items.data(), items.size() * sizeof(Item)));
-        NVD_TRY(up(pl->splits, splits.data(), splits.size() * sizeof(RsSplit)));
-        NVD_TRY(up(pl->tasks, tasks.data(), tasks.size() * sizeof(FillTask)));
-        NVD_TRY(up(pl->node, node.data(), node.size() * 4));
-        NVD_TRY(up(pl->slot_row, slot_row.data(), slot_row.size() * 4));
-        NVD_TRY(up(pl->slot_of, slot_of.data(), slot_of.size() * 4));
-        NVD_TRY(pl->deg.alloc(pl->n_slots * 8));
-        NVD_TRY(pl->dinv.alloc(pl->n_slots * 8));
-        NVD_TRY(pl->col.alloc(std::max<int64_t>(ne, 4) * 4));
-        NVD_TRY(pl->w.alloc(std::max<int64_t>(ne, 4) * 8));
+        add(0, ctas.data(), ctas.size() * sizeof(RsCta));
+        add(1, items.data(), items.size() * sizeof(Item));
+        add(2, splits.data(), splits.size() * sizeof(RsSplit));
+        add(3, tasks.data(), tasks.size() * sizeof(FillTask));
+        add(4, node.data(), node.size() * 4);
+        add(5, slot_row.data(), slot_row.size() * 4);
+        add(6, slot_of.data(), slot_of.size() * 4);
+        NVD_TRY(pl->meta.alloc(host.size()));
+        NVD_TRY_CUDA(cudaMemcpy(pl->meta.p, host.data(), host.size(), cudaMemcpyHostToDevice));
+        char *m = pl->meta.as<char>();
+        pl->ctas = (RsCta *)(m + off[0]);
+        pl->items = (Item *)(m + off[1]);
+        pl->splits = (RsSplit *)(m + off[2]);
+        pl->tasks = (FillTask *)(m + off[3]);
+        pl->node = (int32_t *)(m + off[4]);
+        pl->slot_row = (int32_t *)(m + off[5]);
+        pl->slot_of = (int32_t *)(m + off[6]);
+        // weights, degrees, columns: entries come in multiples of 4 per lane group
+        NVD_TRY(pl->data.alloc((size_t)ne * 12 + (size_t)pl->n_slots * 16 + 64));
+        pl->w = pl->data.as<double>();
+        pl->col = (int32_t *)(pl->w + ne);
+        pl->deg = (double *)(pl->col + ne);
+        pl->dinv = pl->deg + pl->n_slots;
         NVD_TRY(fill_plan(g, pl.get(), 0));
         NVD_TRY_CUDA(cudaDeviceSynchronize());
     }
@@ -692,14 +724,14 @@ int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, co
         const int c0 = t * KT, kc = std::min(KT, k - c0);
         const size_t off = own.idx ? (size_t)c0 * xsz : (size_t)c0 * own.ld * xsz;
         RsArgs a{};
-        a.ctas = pl->ctas.as<RsCta>();
-        a.items = pl->items.as<Item>();
-        a.splits = pl->splits.as<RsSplit>();
-        a.col = pl->col.as<int32_t>();
-        a.w = pl->w.as<double>();
-        a.node = pl->node.as<int32_t>();
-        a.deg = pl->deg.as<double>();
-        a.dinv = pl->dinv.as<double>();
+        a.ctas = pl->ctas;
+        a.items = pl->items;
+        a.splits = pl->splits;
+        a.col = pl->col;
+        a.w = pl->w;
+        a.node = pl->node;
+        a.deg = pl->deg;
+        a.dinv = pl->dinv;
         a.own = own;
         a.own.x = (const char *)own.x + off;
         a.own.y = (const char *)own.y + off;
