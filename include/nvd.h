@@ -225,6 +225,9 @@ typedef struct {
  * use the row split and block count, and nvd_ge_distance uses the tile width
  * when opts.kt = 0 and the launch mode and iteration form when the flags leave
  * them at their defaults.
+ * With NVD_TUNE_SINGLE_RHS in FP64 mode the form an open call takes by itself is
+ * timed too; otherwise a tuned FP64 handle keeps its tiles, and a graph that fits
+ * the one-launch forms (nvd_ge_distance) is better left untuned.
  * Results do not depend on the choice beyond rounding (each choice is a valid
  * order of the same sums).  Synchronous.
  *   k      number of pairs the later calls will solve (sets the tile-width cost
@@ -263,6 +266,14 @@ int nvd_graph_set_tuning(nvd_graph_t g, int32_t mode, const nvd_tune_result *t);
  * variational estimate 2 delta^T z - z^T L z from the FP64 residual (error
  * quadratic in the error of z).  Non-convergence still writes every output and
  * returns NVD_ERR_NOT_CONVERGED; per-pair status is in stats.
+ *
+ * An FP64 solve that leaves its form open (opts kt = 0, no NVD_SOLVE_PERSISTENT,
+ * FOLD_DIRECTION or TEST_TIMEOUT, no tile width or such form chosen by
+ * nvd_graph_tune) runs as one
+ * thread-block cluster per (component, pair), as one cooperative kernel with the
+ * vectors in shared memory (one component, not with NVD_SOLVE_NO_SYNC), or as
+ * host-driven launches over tiles of columns, whichever is estimated to take the
+ * least time on this graph; the stopping rule is the same in all three.
  */
 int nvd_ge_distance(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_t xdtype,
                     const nvd_solve_opts *opts, double *d2_out, void *z_out,
@@ -413,8 +424,10 @@ int nvd_network_variance(nvd_graph_t g, int32_t s, const int32_t *nodes, const d
  * nvd_ge_distance_batched -- many graphs in one solve: the G graphs are treated as
  * the diagonal blocks of one block-diagonal Laplacian and every (graph, pair)
  * keeps its own CG scalars and convergence test, so the result equals G
- * independent nvd_ge_distance calls.  The PCG iterations are driven from the
- * host, one launch per phase over all graphs (the kernels of nvd_ge_distance at
+ * independent nvd_ge_distance calls.  In FP64 mode with kt = 0 and components
+ * that fit, every (component, pair) is solved by one thread-block cluster in a
+ * single launch where that is estimated to be faster (as in nvd_ge_distance).
+ * Otherwise the PCG iterations are driven from the host, one launch per phase over all graphs (the kernels of nvd_ge_distance at
  * full occupancy; convergence polled one batch behind), or, with
  * NVD_SOLVE_PERSISTENT, run inside one persistent cooperative kernel captured in
  * a CUDA graph (replayed when the same arguments come again).  Measured on the

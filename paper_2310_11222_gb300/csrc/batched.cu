@@ -257,7 +257,7 @@ int batched_impl(const nvd_graph_t *gs, int32_t G, const int32_t *k_per, const v
         int cs = 0;
         double us = 0.0;
         NVD_TRY(cluster_estimate(U, kmax, &cs, &us));
-        if (cs && us <= tiles_iter_us(U->n, U->nnz, KT, (kmax + KT - 1) / KT)) NVD_TRY(cluster_plan_get(U, cs, &cpl));
+        if (cs && us <= tiles_iter_us(U->n, U->nnz, KT, (kmax + KT - 1) / KT)) NVD_TRY(unless_oom(cluster_plan_get(U, cs, &cpl)));
         if (cpl) {
             int wst = NVD_OK;
             Owner *d_own = (Owner *)U->wsp("owners", (size_t)G * sizeof(Owner), &wst);

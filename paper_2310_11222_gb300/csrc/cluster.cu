@@ -26,7 +26,8 @@
 // 65 clocks for a dependent multiply-add, 107 for a butterfly step, 650 for a division).
 // With many rows per CTA that rate is the limit -- one multiply-add per entry, 9 operations
 // per row -- and below a few hundred rows the chain of dependent FP64 instructions, so the
-// reductions add across lanes in integers (warp_sum) and spread over the SM's quarters.
+// partial sums of a CTA go through shared memory to a few warps spread over the SM's quarters
+// (cluster_sum) instead of a butterfly in every warp.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -164,9 +165,9 @@ __device__ __forceinline__ void cluster_sum(ClState &st, double *red, int cs, in
 // clocks against 300).
 //
 // Measured, FP64 to 1e-10, whole call (before: the host-driven tiles): one pair on a BA
-// graph of 2,000 nodes 0.25 ms (0.94), 16 pairs 0.32 ms (2.0); one pair on a ring of 20,011
-// 1.2 ms (2.0); 96 graphs of 24..500 nodes, 4 pairs each, 0.47 ms (2.9); 96 node pairs on an
-// ER graph of 30,011 nodes 4.8 ms (18.2).  An iteration at 2,000 nodes and 16 CTAs takes
+// graph of 2,000 nodes 0.22 ms (0.92), 16 pairs 0.27 ms (2.2); one pair on a ring of 20,011
+// 1.1 ms (2.0); 96 graphs of 24..500 nodes, 4 pairs each, 0.59 ms (2.9); 96 node pairs on an
+// ER graph of 30,011 nodes 4.8 ms (18.2; resident.cu 4.1).  An iteration at 2,000 nodes and 16 CTAs takes
 // 13,600 clocks: row sums 3,700, sums 2,900 and 3,400, publishing p 2,900.
 template <bool PG, bool MS, bool ONE>
 __global__ void __launch_bounds__(CL_MAX_NT, 1) k_cluster_pcg(const __grid_constant__ ClArgs a) {

@@ -190,6 +190,8 @@ size_t l2_persist_bytes();
 // 4.0, 32 FP32 columns of a power-law graph of 2 * 10^6 88 ms against 81; with 0.4 of a wave
 // that graph took 121 ms.
 int target_blocks(const nvd_graph_s *g);
+// A status, with OK for "no memory": what is only a faster form is then left out.
+inline int unless_oom(int rc) { return rc == NVD_ERR_OOM ? (int)NVD_OK : rc; }
 // Fresh handle id.
 uint64_t next_graph_id();
 

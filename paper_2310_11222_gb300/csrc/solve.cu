@@ -89,7 +89,8 @@ int check_opts(const nvd_solve_opts &o) {
 // launch-by-launch profiling.  Three estimates of one iteration over all k columns decide:
 // one cluster per (component, pair) (cluster.cu), one persistent kernel with the vectors on
 // chip (resident.cu, the tile width of the least time), the host-driven tiles.  Host inputs
-// of the on-chip forms are staged whole, so only up to 256 MB of them.
+// of the on-chip forms are staged whole, so only up to 256 MB of them.  A plan that finds no
+// memory leaves the solve to the tiles.
 int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size_t in_bytes, bool warm,
                 ClusterPlan **cluster, ResidentPlan **resident) {
     *cluster = nullptr;
@@ -110,14 +111,14 @@ int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size
             if (kt > KT && kt > 1) break;
             us = ((k + kt - 1) / kt) * resident_iter_us(g->h_seg_end[0] - g->h_seg_begin[0], g->nnz, kt);
             ResidentPlan *pl = nullptr;
-            if (us < best) NVD_TRY(resident_plan_for(g, kt, &pl));
+            if (us < best) NVD_TRY(unless_oom(resident_plan_for(g, kt, &pl)));
             if (pl) {
                 best = us;
                 rkt = kt;
                 *resident = pl;
             }
         }
-    if (!rkt && cs) NVD_TRY(cluster_plan_get(g, cs, cluster));
+    if (!rkt && cs) NVD_TRY(unless_oom(cluster_plan_get(g, cs, cluster)));
     return NVD_OK;
 }
 
@@ -126,7 +127,8 @@ int onchip_distance(nvd_graph_t g, ClusterPlan *cpl, ResidentPlan *rpl, const nv
                      int32_t xdt, double *d2_out, void *z_out, nvd_solve_stats *stats, cudaStream_t s, bool idx) {
     const size_t xsz = xdt == NVD_F64 ? 8 : 4, bytes = (size_t)k * g->n * xsz;
     const bool host_in = o.flags & NVD_SOLVE_HOST_INPUTS, d2_dev = o.flags & NVD_SOLVE_D2_DEVICE;
-    const bool want = !d2_dev || stats || host_in || rpl;
+    const bool report = !d2_dev || stats || host_in;   // per-pair results go back to the caller
+    const bool want = report || rpl;
     int st = NVD_OK;
     void *z = z_out;
     double *d2 = d2_dev ? d2_out : nullptr;
@@ -147,7 +149,7 @@ int onchip_distance(nvd_graph_t g, ClusterPlan *cpl, ResidentPlan *rpl, const nv
     if (host_in && z_out) NVD_TRY_CUDA(cudaMemcpyAsync(z_out, z, bytes, cudaMemcpyDeviceToHost, s));
     if (!(o.flags & NVD_SOLVE_NO_SYNC) || want) NVD_TRY_CUDA(cudaStreamSynchronize(s));
     int overall = NVD_OK;
-    if (want)
+    if (report)
         for (int32_t j = 0; j < k; ++j) {
             const ColResult &r = res[j];
             if (!d2_dev) d2_out[j] = r.d2;

@@ -1,6 +1,8 @@
 """FP64 solves by one persistent kernel with the vectors on chip: every tile width with ragged
 last tiles, rows split over several warps, x in shared or global memory, and the call forms,
 against the oracle and the tiled solve."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -139,3 +141,18 @@ def test_tiled_rows_over_all_lane_groups(nvd, case, kt):
     d32 = nvd.ge_distance(nvd.Graph(g.rowptr, g.colidx, w32), on(X[:9]), on(Y[:9]), rtol=1e-11, kt=kt).cpu().numpy()
     ref = ocg.ge_d2_cg(g.n, g.rowptr, g.colidx, w32.astype(np.float64), X[:9], Y[:9], rtol=1e-13)[0]
     assert rel(d32, ref) < 1e-10
+
+
+# device d^2 and no stats: nobody asks for the pairs' statuses, in either form of the solve
+@pytest.mark.parametrize("kt", [0, 4])
+def test_device_result_without_statuses(nvd, case, kt):
+    g, X, Y, _ = case
+    k = 6
+    G = nvd.Graph.from_csr(g)
+    x, y = on(X[:k]), on(Y[:k])
+    d2 = torch.full((k,), np.nan, dtype=torch.float64, device=DEV)
+    o = nvd.default_opts(nvd.MODE_FP64, max_iter=3, kt=kt)
+    o.flags |= nvd.SOLVE_D2_DEVICE
+    rc = nvd.load_library().nvd_ge_distance(G.handle, k, x.data_ptr(), y.data_ptr(), nvd.F64, ctypes.byref(o),
+                                            d2.data_ptr(), None, None, torch.cuda.current_stream().cuda_stream)
+    assert rc == 0 and bool(torch.isfinite(d2).all())
