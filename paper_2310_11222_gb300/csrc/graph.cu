@@ -689,8 +689,17 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
         most_rows = std::max(most_rows, nr);
         heavy_blocks += (seg_item_off[s + 1] - seg_item_off[s] + (int64_t)heavy_per - 1) / (int64_t)heavy_per;
     }
-    if (10 * most_rows < 9 * seg_rows) heavy_blocks = 0;
-    const int wave = (tma ? 2 : 1) * target_blocks(g) * std::max(g->sp.blocks_pct, 100) / 100;
+    // Where no component has nearly all rows, blocks in order gather from a few components at
+    // a time: a wave of them for every 22 MB of the gathered vector, up to four, keeps what a wave gathers
+    // in L2 beside its streams.  Batches of graphs, one wave against this many, ms per solve:
+    // 64 of 10^3..2 * 10^5 nodes (220 MB) 32 columns FP32 29.0 and 20.9, 16 FP64 142 and 114; 0.3 times
+    // as large (66 MB) 8.5 and 7.4, 44.4 and 38.0; a tenth (22 MB) 3.4 with one, about 10% more with two.
+    int waves = tma ? 2 : 1;
+    if (10 * most_rows < 9 * seg_rows) {
+        heavy_blocks = 0;
+        if (!tma) waves = (int)std::min<int64_t>(4, std::max<int64_t>(1, seg_rows * KT * szv / 22000000));
+    }
+    const int wave = waves * target_blocks(g) * std::max(g->sp.blocks_pct, 100) / 100;
     const int T = std::max<int>(1, wave - (heavy_blocks <= wave / 4 ? (int)std::min<int64_t>(heavy_blocks, wave / 10) : 0));
     const double target = ltot / T;
     // block sizes in whole slices (warps take a block's slices as they free up)
