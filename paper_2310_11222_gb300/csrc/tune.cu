@@ -69,6 +69,8 @@ struct Bench {
 
     bool fold = false;     // time the two-kernel iteration
 
+    bool open = false;     // single right-hand sides in the form an open call takes (KT: how many)
+
     // One solve of KT columns, max_iter = iters; returns its device time in ms.
     int run(int KT, bool persistent, int iters, float *ms) {
         nvd_solve_opts o;
@@ -76,9 +78,9 @@ struct Bench {
         o.mode = mode;
         o.rtol = 1e-300;            // never met: every column runs max_iter iterations
         o.max_iter = iters;
-        o.kt = KT;
+        o.kt = open ? 0 : KT;
         o.check_every = 4;
-        o.flags = NVD_SOLVE_D2_DEVICE | (KT == 1 ? NVD_SOLVE_SINGLE_RHS : 0u) |
+        o.flags = NVD_SOLVE_D2_DEVICE | (open || KT == 1 ? NVD_SOLVE_SINGLE_RHS : 0u) |
                   (persistent ? NVD_SOLVE_PERSISTENT : 0u) | (fold ? NVD_SOLVE_FOLD_DIRECTION : 0u);
         NVD_TRY_CUDA(cudaEventRecord(t.a, s));
         const int rc = ge_distance_internal(g, KT, x, y, NVD_F64, &o, d2, s);
@@ -302,6 +304,23 @@ int tune_impl(nvd_graph_s *g, int32_t mode, int32_t k, uint32_t flags, nvd_tune_
             best_iter = alt;
         } else {
             best_iter = std::min(best_iter, base);
+        }
+    }
+    // 6. single right-hand sides in FP64: the form an open call takes by itself (one launch
+    //    with the vectors on chip where that is estimated to be faster), all of them in one
+    //    call, against the best tile one after the other.  One pair on 1,000..10^5 nodes of
+    //    mean degree 8, whole call: ER 0.60 to 0.19, 0.66 to 0.31, 0.90 to 0.46 ms.
+    if (single && mode == NVD_MODE_FP64) {
+        const int cols = std::min(k, 32);
+        double it = INFINITY;
+        b.open = true;
+        const int rc = b.per_iter(cols, false, &it);
+        b.open = false;
+        if (rc) return fail(rc);
+        ++ntried;
+        if (it < cols * best_iter * 0.97) {
+            pers = fold = 0;
+            best_iter = it / cols;
         }
     }
     restore_timed();
