@@ -431,10 +431,10 @@ int nvd_network_variance(nvd_graph_t g, int32_t s, const int32_t *nodes, const d
  * full occupancy; convergence polled one batch behind), or, with
  * NVD_SOLVE_PERSISTENT, run inside one persistent cooperative kernel captured in
  * a CUDA graph (replayed when the same arguments come again).  Measured on the
- * 64-graph workload (1.7e6 nodes) the host-driven form takes 23 ms per FP32 step
- * against 45 ms; the persistent kernel (two CTAs per SM at its register count,
- * three grid barriers per iteration) is ahead by at most ~10% on batches of a few
- * graphs or a few tens of thousands of nodes.
+ * 64-graph workload (1.7e6 nodes) the host-driven form takes 21 ms per FP32 step
+ * against 43 ms; the persistent kernel (two CTAs per SM at its register count,
+ * three grid barriers per iteration) is behind on smaller batches too (8 graphs of
+ * 104,010 nodes 2.0 against 2.6 ms).
  *
  *   graphs  [G] handles (same device).
  *   k_per   [G] pairs per graph.
