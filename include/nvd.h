@@ -269,8 +269,7 @@ int nvd_graph_set_tuning(nvd_graph_t g, int32_t mode, const nvd_tune_result *t);
  *
  * An FP64 solve that leaves its form open (opts kt = 0, no NVD_SOLVE_PERSISTENT,
  * FOLD_DIRECTION or TEST_TIMEOUT, no tile width or such form chosen by
- * nvd_graph_tune) runs as one
- * thread-block cluster per (component, pair), as one cooperative kernel with the
+ * nvd_graph_tune) runs as one thread-block cluster per (component, pair), as one cooperative kernel with the
  * vectors in shared memory (one component, not with NVD_SOLVE_NO_SYNC), or as
  * host-driven launches over tiles of columns, whichever is estimated to take the
  * least time on this graph; the stopping rule is the same in all three.
@@ -427,8 +426,8 @@ int nvd_network_variance(nvd_graph_t g, int32_t s, const int32_t *nodes, const d
  * independent nvd_ge_distance calls.  In FP64 mode with kt = 0 and components
  * that fit, every (component, pair) is solved by one thread-block cluster in a
  * single launch where that is estimated to be faster (as in nvd_ge_distance).
- * Otherwise the PCG iterations are driven from the host, one launch per phase over all graphs (the kernels of nvd_ge_distance at
- * full occupancy; convergence polled one batch behind), or, with
+ * Otherwise the PCG iterations are driven from the host, one launch per phase
+ * over all graphs (the kernels of nvd_ge_distance at full occupancy; convergence polled one batch behind), or, with
  * NVD_SOLVE_PERSISTENT, run inside one persistent cooperative kernel captured in
  * a CUDA graph (replayed when the same arguments come again).  Measured on the
  * 64-graph workload (1.7e6 nodes) the host-driven form takes 21 ms per FP32 step
