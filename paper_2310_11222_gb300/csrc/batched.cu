@@ -251,8 +251,10 @@ int batched_impl(const nvd_graph_t *gs, int32_t G, const int32_t *k_per, const v
     }
     const size_t szv = o.mode == NVD_MODE_FP64 ? 8 : 4;
     const size_t xsz = xdt == NVD_F64 ? 8 : 4;
-    if (o.mode == NVD_MODE_FP64 && !o.kt && !(o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION))) {
-        // one cluster per (graph, component, pair) where that is faster (cluster.cu)
+    if (o.mode == NVD_MODE_FP64 && !o.kt && !(o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION)) &&
+        !prof_enabled()) {
+        // one cluster per (graph, component, pair) where that is faster (cluster.cu); its one
+        // launch has no SpMV launches for the kernel timing to bracket
         ClusterPlan *cpl = nullptr;
         int cs = 0;
         double us = 0.0;
