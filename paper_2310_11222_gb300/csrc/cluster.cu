@@ -854,6 +854,12 @@ int cluster_plan_get(nvd_graph_s *g, int cs, ClusterPlan **out) {
     return NVD_OK;
 }
 
+void cluster_variant(const ClusterPlan *pl, int32_t *cs, int32_t *variant) {
+    const ClClass &c = pl->classes.front();
+    *cs = c.cs;
+    *variant = (c.pg ? 1 : 0) | (c.ms ? 2 : 0) | (c.one ? 4 : 0) | (c.l2 ? 8 : 0);
+}
+
 int cluster_refill(nvd_graph_s *g, cudaStream_t s) {
     if (!g->clusters) return NVD_OK;
     for (auto &kv : g->clusters->plans) NVD_TRY(fill_cluster_plan(g, kv.second.get(), s));

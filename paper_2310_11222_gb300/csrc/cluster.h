@@ -12,6 +12,9 @@ struct ClusterPlan;
 int cluster_estimate(nvd_graph_s *g, int64_t cols, int *cs, double *us);
 // The plan for that cluster size (after cluster_estimate), or *out = NULL if it does not fit.
 int cluster_plan_get(nvd_graph_s *g, int cs, ClusterPlan **out);
+// The largest component's cluster size and kernel variant: 1 p gathered from L2, 2 matrix in
+// shared memory, 4 one slot per thread, 8 p published through L2.
+void cluster_variant(const ClusterPlan *pl, int32_t *cs, int32_t *variant);
 // Estimated microseconds of one iteration of the host-driven loop on `tiles` tiles of kt FP64
 // columns, fitted to runs from 3 * 10^4 to 10^6 rows: three launches and their block reductions,
 // and 1.35 times the FP64 instructions (a multiply-add per entry and 10 operations per row, at 2

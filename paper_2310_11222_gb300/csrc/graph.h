@@ -111,6 +111,11 @@ void resident_state_delete(ResidentState *c);
 int64_t resident_state_bytes(const ResidentState *c);
 }  // namespace nvd
 
+namespace nvd {
+// Forms of an FP64 solve (pick_onchip, solve.cu).
+enum SolveForm : int32_t { FORM_OPEN = 0, FORM_TILES = 1, FORM_CLUSTER = 2, FORM_RESIDENT = 3 };
+}  // namespace nvd
+
 struct nvd_graph_s {
     uint64_t id = 0;             // unique per handle (cache keys)
     int device = 0;
@@ -153,6 +158,10 @@ struct nvd_graph_s {
     std::unique_ptr<nvd::ClusterState, void (*)(nvd::ClusterState *)> clusters{nullptr, nvd::cluster_state_delete};
     // plans of the solve with the vectors on chip (one component, FP64)
     std::unique_ptr<nvd::ResidentState, void (*)(nvd::ResidentState *)> resident{nullptr, nvd::resident_state_delete};
+    // for the tests (nvd_diag_*, solve.cu): the form every open FP64 solve takes with its width
+    // (CTAs per cluster or columns per tile), and the form, width and kernel variant of the last one
+    int32_t force_form = nvd::FORM_OPEN, force_width = 0;
+    int32_t last_form = nvd::FORM_OPEN, last_width = 0, last_variant = 0;
     ~nvd_graph_s();
 
     void *wsp(const std::string &name, size_t bytes, int *st);

@@ -698,6 +698,9 @@ int resident_plan_for(nvd_graph_s *g, int KT, ResidentPlan **out) {
     return NVD_OK;
 }
 
+int32_t resident_width(const ResidentPlan *pl) { return pl->KT; }
+int32_t resident_variant(const ResidentPlan *pl) { return pl->x_global ? 1 : 0; }
+
 int resident_refill(nvd_graph_s *g, cudaStream_t s) {
     if (!g->resident) return NVD_OK;
     for (auto &kv : g->resident->plans)

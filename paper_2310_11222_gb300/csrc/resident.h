@@ -14,6 +14,10 @@ double resident_iter_us(int64_t n, int64_t nnz, int KT);
 // isolated nodes), its vectors do not fit, or KT is not 1, 4, 8 or 16.
 int resident_plan_for(nvd_graph_s *g, int KT, ResidentPlan **out);
 
+// Columns per tile of a plan, and its kernel variant: 1 x in global memory.
+int32_t resident_width(const ResidentPlan *pl);
+int32_t resident_variant(const ResidentPlan *pl);
+
 // Solve k columns, tile after tile (own: x, y, z at column 0).  d2dev: [k] device or NULL.
 // want_res: read the [k] results back (synchronises s) into a buffer of the handle, valid
 // until its next solve; without it a bounded wait that gave up goes unreported.

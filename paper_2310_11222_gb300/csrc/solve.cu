@@ -98,8 +98,18 @@ int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size
     if (o.mode != NVD_MODE_FP64 || o.kt || warm || prof_enabled() || g->tuned_kt[o.mode] ||
         g->tuned_persistent[o.mode] || g->tuned_fold[o.mode] ||
         (o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION | NVD_SOLVE_TEST_TIMEOUT)) ||
-        ((o.flags & NVD_SOLVE_HOST_INPUTS) && 2 * in_bytes > ((size_t)1 << 28)))
+        ((o.flags & NVD_SOLVE_HOST_INPUTS) && 2 * in_bytes > ((size_t)1 << 28)) || g->force_form == FORM_TILES)
         return NVD_OK;
+    if (g->force_form) {   // (the estimate sets up what a cluster plan needs)
+        int cs = 0;
+        double us = 0.0;
+        NVD_TRY(cluster_estimate(g, k, &cs, &us));
+        if (g->force_form == FORM_RESIDENT) NVD_TRY(resident_plan_for(g, g->force_width, resident));
+        else if (cs) NVD_TRY(cluster_plan_get(g, g->force_width, cluster));
+        if (*resident || *cluster) return NVD_OK;
+        set_error("the form asked for does not fit the graph");
+        return NVD_ERR_UNSUPPORTED;
+    }
     double best = tiles_iter_us(g->n, g->nnz, KT, (k + KT - 1) / KT), us = 0.0;
     int cs = 0, rkt = 0;
     NVD_TRY(cluster_estimate(g, k, &cs, &us));
@@ -143,6 +153,13 @@ int onchip_distance(nvd_graph_t g, ClusterPlan *cpl, ResidentPlan *rpl, const nv
     }
     if (z && g->n_singleton > 0) NVD_TRY_CUDA(cudaMemsetAsync(z, 0, bytes, s));
     const Owner own{x, y, z, 0, g->n, k, 0, g->nseg, idx ? 1 : 0};
+    g->last_form = rpl ? FORM_RESIDENT : FORM_CLUSTER;
+    if (rpl) {
+        g->last_width = resident_width(rpl);
+        g->last_variant = resident_variant(rpl);
+    } else {
+        cluster_variant(cpl, &g->last_width, &g->last_variant);
+    }
     ColResult *res = nullptr;
     if (rpl) NVD_TRY(resident_solve(g, rpl, o, own, k, xdt, d2, want, &res, s));
     else NVD_TRY(cluster_solve(g, cpl, o, nullptr, own, 1, k, xdt, z != nullptr, d2, want, &res, s));
@@ -195,6 +212,9 @@ int distance_impl(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_
         NVD_TRY(pick_onchip(g, o, k, KT, (size_t)k * g->n * (xdt == NVD_F64 ? 8 : 4), z0 != nullptr, &cpl, &rpl));
         if (cpl || rpl) return onchip_distance(g, cpl, rpl, o, k, x, y, xdt, d2_out, z_out, stats, s, idx);
     }
+    g->last_form = FORM_TILES;
+    g->last_width = KT;
+    g->last_variant = 0;
     const bool mixed = o.mode == NVD_MODE_MIXED;
     const size_t szv = o.mode == NVD_MODE_FP64 ? 8 : 4;
     const size_t xsz = xdt == NVD_F64 ? 8 : 4;
@@ -900,4 +920,31 @@ extern "C" int nvd_laplacian_apply(nvd_graph_t g, int32_t k, const void *x, void
         set_error("nvd_laplacian_apply: unexpected host exception");
         return NVD_ERR_CUDA;
     }
+}
+
+// For the package's tests, not part of nvd.h: make every open FP64 solve of the handle take a
+// form (nvd::SolveForm; FORM_OPEN: by estimate again) of that width, and read the form, width
+// and kernel variant (cluster_variant, resident_variant) of the last solve.
+extern "C" int nvd_diag_force_form(nvd_graph_t g, int32_t form, int32_t width) {
+    clear_error();
+    if (!g || form < FORM_OPEN || form > FORM_RESIDENT || (form == FORM_CLUSTER && !(width == 1 || width == 2 ||
+        width == 4 || width == 8 || width == 16))) {
+        set_error("nvd_diag_force_form: invalid argument");
+        return NVD_ERR_INVALID_ARG;
+    }
+    g->force_form = form;
+    g->force_width = width;
+    return NVD_OK;
+}
+
+extern "C" int nvd_diag_last_form(nvd_graph_t g, int32_t *form, int32_t *width, int32_t *variant) {
+    clear_error();
+    if (!g || !form || !width || !variant) {
+        set_error("nvd_diag_last_form: invalid argument");
+        return NVD_ERR_INVALID_ARG;
+    }
+    *form = g->last_form;
+    *width = g->last_width;
+    *variant = g->last_variant;
+    return NVD_OK;
 }
