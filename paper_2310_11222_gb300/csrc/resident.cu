@@ -79,6 +79,7 @@ struct RsArgs {
     double *d2dev;             // [kc] or NULL
     double rtol2, d2stop;
     int32_t max_iter, xdt, write_z;
+    int32_t bar_extra;         // arrivals a meeting waits for beyond the grid's (NVD_SOLVE_TEST_TIMEOUT)
 };
 
 // Scalars per column, the same in every CTA.
@@ -110,7 +111,7 @@ __device__ __forceinline__ bool grid_meet(const RsArgs &a, RsState &st, unsigned
         const uint64_t t0 = timer_ns();
         for (unsigned spin = 1;; ++spin) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.bar) : "memory");
-            if ((int)(seen - target) >= 0) break;
+            if ((int)(seen - target) >= a.bar_extra) break;
             if ((spin & 1023u) == 0 && (__ldcg(a.err) != 0 || timer_ns() - t0 > 2000000000ull)) {
                 atomicCAS(a.err, 0, (int)NVD_ERR_TIMEOUT);
                 st.fail = 1;
@@ -753,6 +754,7 @@ int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, co
         a.max_iter = o.max_iter;
         a.xdt = xdt == NVD_F64 ? 1 : 0;
         a.write_z = own.z ? 1 : 0;
+        a.bar_extra = (o.flags & NVD_SOLVE_TEST_TIMEOUT) ? 1 : 0;
         switch (KT) {
             case 1: NVD_TRY(launch<1>(pl, a, s)); break;
             case 4: NVD_TRY(launch<4>(pl, a, s)); break;

@@ -97,7 +97,9 @@ int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size
     *resident = nullptr;
     if (o.mode != NVD_MODE_FP64 || o.kt || warm || prof_enabled() || g->tuned_kt[o.mode] ||
         g->tuned_persistent[o.mode] || g->tuned_fold[o.mode] ||
-        (o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION | NVD_SOLVE_TEST_TIMEOUT)) ||
+        (o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION)) ||
+        // (the timeout test reaches only the form with a grid barrier, and that only when forced)
+        ((o.flags & NVD_SOLVE_TEST_TIMEOUT) && g->force_form != FORM_RESIDENT) ||
         ((o.flags & NVD_SOLVE_HOST_INPUTS) && 2 * in_bytes > ((size_t)1 << 28)) || g->force_form == FORM_TILES)
         return NVD_OK;
     if (g->force_form) {   // (the estimate sets up what a cluster plan needs)

@@ -3,6 +3,7 @@ it, so that what runs here does not depend on the estimates that choose a form: 
 width of the one-kernel form with several tiles and a ragged last one, every kernel of the
 cluster form, new weights, and the call forms, against the oracle."""
 import ctypes
+import time
 
 import numpy as np
 import pytest
@@ -160,3 +161,25 @@ def test_open_calls_take_the_estimated_form(nvd, case):
     force(nvd, G, 0, 0)
     nvd.ge_distance(G, x, y)
     assert last(nvd, G)[0] == CLUSTER
+
+
+def test_one_kernel_wait_that_gives_up(nvd, case):
+    """The grid meeting waits for one arrival more than the grid has, so its bounded wait (2 s)
+    runs out in the first of three tiles: one NVD_ERR_TIMEOUT for the call, the later tiles leave
+    at once, and the next solve on the handle is right."""
+    g, X, Y, want = case
+    G = nvd.Graph.from_csr(g)
+    force(nvd, G, RESIDENT, 8)
+    d2 = nvd.ge_distance(G, on(X), on(Y), rtol=1e-11)
+    t0 = time.perf_counter()
+    with pytest.raises(nvd.NvdError) as e:
+        nvd.ge_distance(G, on(X), on(Y), rtol=1e-11, test_timeout=True)
+    dt = time.perf_counter() - t0
+    assert e.value.status == 8 and last(nvd, G)[:2] == (RESIDENT, 8)
+    assert 1.5 < dt < 3.5                                # one wait of 2 s, not one per tile
+    again = nvd.ge_distance(G, on(X), on(Y), rtol=1e-11)
+    assert torch.equal(d2, again) and rel(again.cpu().numpy(), want) < 1e-10
+    # an open call with the flag keeps the tiles, which have no such wait
+    force(nvd, G, 0, 0)
+    t = nvd.ge_distance(G, on(X), on(Y), rtol=1e-11, test_timeout=True).cpu().numpy()
+    assert last(nvd, G)[0] == TILES and rel(t, want) < 1e-10
