@@ -272,7 +272,8 @@ int nvd_graph_set_tuning(nvd_graph_t g, int32_t mode, const nvd_tune_result *t);
  * nvd_graph_tune) runs as one thread-block cluster per (component, pair), as one cooperative kernel with the
  * vectors in shared memory (one component, not with NVD_SOLVE_NO_SYNC), or as
  * host-driven launches over tiles of columns, whichever is estimated to take the
- * least time on this graph; the stopping rule is the same in all three.
+ * least time on this graph; the stopping rule is the same in all three.  Where the first two
+ * find no memory for their plan or workspace the tiles, which need less, take the solve.
  */
 int nvd_ge_distance(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_t xdtype,
                     const nvd_solve_opts *opts, double *d2_out, void *z_out,

@@ -241,6 +241,7 @@ int batched_impl(const nvd_graph_t *gs, int32_t G, const int32_t *k_per, const v
     UnionGraph *u = nullptr;
     NVD_TRY(get_union(gs, G, s, &u));
     nvd_graph_s *U = u->g.get();
+    U->alloc_limit = gs[0]->alloc_limit;
     int KT = o.kt;
     if (!KT) {
         const int cap = o.mode == NVD_MODE_FP64 ? 16 : 32;
@@ -261,30 +262,36 @@ int batched_impl(const nvd_graph_t *gs, int32_t G, const int32_t *k_per, const v
         NVD_TRY(cluster_estimate(U, kmax, &cs, &us));
         if (cs && us <= tiles_iter_us(U->n, U->nnz, KT, (kmax + KT - 1) / KT)) NVD_TRY(unless_oom(cluster_plan_get(U, cs, &cpl)));
         if (cpl) {
-            int wst = NVD_OK;
-            Owner *d_own = (Owner *)U->wsp("owners", (size_t)G * sizeof(Owner), &wst);
-            if (wst) return wst;
-            std::vector<Owner> own(G);
-            std::vector<int64_t> off(G + 1, 0);
-            for (int i = 0; i < G; ++i) {
-                own[i] = Owner{x[i], y[i], nullptr, u->node_off[i], gs[i]->n, k_per[i], u->seg_off[i], u->seg_off[i + 1], 0};
-                off[i + 1] = off[i] + k_per[i];
-            }
-            NVD_TRY_CUDA(cudaMemcpyAsync(d_own, own.data(), G * sizeof(Owner), cudaMemcpyHostToDevice, s));
+            int rc = NVD_OK;
             ColResult *res = nullptr;
-            NVD_TRY(cluster_solve(U, cpl, o, d_own, own[0], G, kmax, xdt, false, nullptr, true, &res, s));
-            int overall = NVD_OK;
-            for (int i = 0; i < G; ++i)
-                for (int j = 0; j < k_per[i]; ++j) {
-                    const ColResult &r = res[(size_t)i * kmax + j];
-                    d2_out[off[i] + j] = r.d2;
-                    if (r.status != NVD_OK && overall != NVD_ERR_NUMERIC) overall = r.status;
-                    if (stats)
-                        stats[off[i] + j] = nvd_solve_stats{
-                            r.iters, 0, r.rr0 > 0.0 ? std::sqrt(std::max(r.rr, 0.0) / r.rr0) : 0.0, r.status, 0};
-                }
-            if (overall != NVD_OK) set_error("nvd_ge_distance_batched: some pair ended with status %d", overall);
-            return overall;
+            std::vector<int64_t> off(G + 1, 0);
+            for (int i = 0; i < G; ++i) off[i + 1] = off[i] + k_per[i];
+            Owner *d_own = (Owner *)U->wsp("owners", (size_t)G * sizeof(Owner), &rc);
+            if (rc == NVD_OK) {
+                std::vector<Owner> own(G);
+                for (int i = 0; i < G; ++i)
+                    own[i] = Owner{x[i], y[i], nullptr, u->node_off[i], gs[i]->n, k_per[i], u->seg_off[i],
+                                   u->seg_off[i + 1], 0};
+                NVD_TRY_CUDA(cudaMemcpyAsync(d_own, own.data(), G * sizeof(Owner), cudaMemcpyHostToDevice, s));
+                rc = cluster_solve(U, cpl, o, d_own, own[0], G, kmax, xdt, false, nullptr, true, &res, s);
+            }
+            if (rc != NVD_ERR_OOM) {
+                if (rc != NVD_OK) return rc;
+                int overall = NVD_OK;
+                for (int i = 0; i < G; ++i)
+                    for (int j = 0; j < k_per[i]; ++j) {
+                        const ColResult &r = res[(size_t)i * kmax + j];
+                        d2_out[off[i] + j] = r.d2;
+                        if (r.status != NVD_OK && overall != NVD_ERR_NUMERIC) overall = r.status;
+                        if (stats)
+                            stats[off[i] + j] = nvd_solve_stats{
+                                r.iters, 0, r.rr0 > 0.0 ? std::sqrt(std::max(r.rr, 0.0) / r.rr0) : 0.0, r.status, 0};
+                    }
+                if (overall != NVD_OK) set_error("nvd_ge_distance_batched: some pair ended with status %d", overall);
+                return overall;
+            }
+            clear_error();   // nothing was launched: the tiles need less
+            U->drop_onchip();
         }
     }
     Plan *pl = nullptr;

@@ -873,74 +873,98 @@ int cluster_solve(nvd_graph_s *g, ClusterPlan *pl, const nvd_solve_opts &o, cons
     int st = NVD_OK;
     const bool direct = n_owner == 1 && g->nseg == 1;
     const size_t nres = (size_t)n_owner * K;
-    ColResult *part = (ColResult *)g->wsp("cl_part", (size_t)std::max(g->nseg, 1) * K * sizeof(ColResult), &st);
-    ColResult *out = direct ? part : (ColResult *)g->wsp("cl_res", nres * sizeof(ColResult), &st);
+    // A graph's columns are solved so many at a time that the results per (component, column)
+    // stay within 64 MB: with node-id inputs they would outgrow everything else (10^5
+    // components and pairs: 320 GB).  Batches (a table of owners) bring vectors of at least that size.
+    const int64_t per_col = (int64_t)std::max(g->nseg, 1) * (int64_t)sizeof(ColResult);
+    const int Kc = owners_dev ? K : (int)std::max<int64_t>(1, std::min<int64_t>(K, ((int64_t)64 << 20) / per_col));
+    ColResult *out = (ColResult *)g->wsp("cl_res", nres * sizeof(ColResult), &st);
+    ColResult *part = direct ? nullptr : (ColResult *)g->wsp("cl_part", (size_t)per_col * Kc, &st);
     if (st) return st;
-    for (const ClClass &cl : pl->classes) {
-        const int64_t tasks = cl.nseg * K;
-        int64_t per = tasks;
-        double *pg = nullptr;
+    // p of the tasks of one launch, up to 256 MB; where there is no memory for that, fewer tasks
+    double *pg = nullptr;
+    int64_t room = 0, want = 0, least = 0;
+    for (const ClClass &cl : pl->classes)
         if (cl.l2) {
-            per = std::max<int64_t>(1, std::min<int64_t>(tasks, ((int64_t)1 << 28) / (8 * cl.max_slots)));
-            pg = (double *)g->wsp("cl_p", (size_t)per * cl.max_slots * 8, &st);
-            if (st) return st;
+            want = std::max(want, cl.nseg * Kc * 8 * cl.max_slots);
+            least = std::max(least, 8 * cl.max_slots);
         }
-        per = std::min<int64_t>(per, ((int64_t)1 << 30) / cl.cs);
-        for (int64_t t0 = 0; t0 < tasks; t0 += per) {
-            ClArgs a{};
-            a.segs = pl->segs.as<ClSeg>() + cl.seg0;
-            a.ctas = pl->ctas.as<ClCta>();
-            a.items = pl->items.as<Item>();
-            a.col = pl->col.as<int32_t>();
-            a.w = pl->w.as<double>();
-            a.node = pl->node.as<int32_t>();
-            a.deg = pl->deg.as<double>();
-            a.dinv = pl->dinv.as<double>();
-            a.owners = owners_dev;
-            a.own0 = own0;
-            a.K = K;
-            a.task0 = t0;
-            a.pg = pg;
-            a.pg_stride = cl.max_slots;
-            a.part = part;
-            a.d2dev = direct ? d2dev : nullptr;
-            a.rtol2 = o.rtol * o.rtol;
-            a.d2stop = (o.flags & NVD_SOLVE_D2_STOP) ? o.d2_rtol : 0.0;
-            a.max_iter = o.max_iter;
-            a.xdt = xdt == NVD_F64 ? 1 : 0;
-            a.write_z = write_z ? 1 : 0;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)(std::min<int64_t>(per, tasks - t0) * cl.cs));
-            cfg.blockDim = dim3(cl.nt);
-            cfg.dynamicSmemBytes = cl.smem;
-            cfg.stream = s;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = cl.cs;
-            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            auto kern = cl.pg ? k_cluster_pcg<true, false, false>
-                        : cl.one ? (cl.ms ? k_cluster_pcg<false, true, true> : k_cluster_pcg<false, false, true>)
-                                 : (cl.ms ? k_cluster_pcg<false, true, false> : k_cluster_pcg<false, false, false>);
-            NVD_TRY_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
-            note_launch(1);
+    if (least) {
+        room = std::max(least, std::min<int64_t>(want, (int64_t)1 << 28));
+        while (!(pg = (double *)g->wsp("cl_p", (size_t)room, &st))) {
+            if (st != NVD_ERR_OOM || room == least) return st;
+            clear_error();
+            st = NVD_OK;
+            room = std::max(least, room / 4);
         }
     }
-    if (!direct) {
-        k_cluster_collect<<<(unsigned)((nres + 127) / 128), 128, 0, s>>>(part, owners_dev, own0, n_owner, K, out,
-                                                                         d2dev);
-        note_launch(1);
-        NVD_TRY_CUDA(cudaGetLastError());
+    if (want_res) NVD_TRY(pinned_results(&cst->h_res, &cst->h_cap, nres));
+    const size_t xsz = own0.idx ? 4 : xdt == NVD_F64 ? 8 : 4, zsz = xdt == NVD_F64 ? 8 : 4;
+    for (int c0 = 0; c0 < K; c0 += Kc) {
+        const int kc = std::min(Kc, K - c0);
+        Owner own = own0;
+        if (c0) {
+            const size_t off = own.idx ? (size_t)c0 * xsz : (size_t)c0 * own.ld * xsz;
+            own.x = (const char *)own.x + off;
+            own.y = (const char *)own.y + off;
+            if (own.z) own.z = (char *)own.z + (size_t)c0 * own.ld * zsz;
+        }
+        if (!owners_dev) own.kc = kc;
+        ColResult *po = direct ? out + c0 : part;
+        for (const ClClass &cl : pl->classes) {
+            const int64_t tasks = cl.nseg * kc;
+            int64_t per = std::min<int64_t>(tasks, ((int64_t)1 << 30) / cl.cs);
+            if (cl.l2) per = std::max<int64_t>(1, std::min<int64_t>(per, room / (8 * cl.max_slots)));
+            for (int64_t t0 = 0; t0 < tasks; t0 += per) {
+                ClArgs a{};
+                a.segs = pl->segs.as<ClSeg>() + cl.seg0;
+                a.ctas = pl->ctas.as<ClCta>();
+                a.items = pl->items.as<Item>();
+                a.col = pl->col.as<int32_t>();
+                a.w = pl->w.as<double>();
+                a.node = pl->node.as<int32_t>();
+                a.deg = pl->deg.as<double>();
+                a.dinv = pl->dinv.as<double>();
+                a.owners = owners_dev;
+                a.own0 = own;
+                a.K = kc;
+                a.task0 = t0;
+                a.pg = cl.l2 ? pg : nullptr;
+                a.pg_stride = cl.max_slots;
+                a.part = po;
+                a.d2dev = direct && d2dev ? d2dev + c0 : nullptr;
+                a.rtol2 = o.rtol * o.rtol;
+                a.d2stop = (o.flags & NVD_SOLVE_D2_STOP) ? o.d2_rtol : 0.0;
+                a.max_iter = o.max_iter;
+                a.xdt = xdt == NVD_F64 ? 1 : 0;
+                a.write_z = write_z ? 1 : 0;
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)(std::min<int64_t>(per, tasks - t0) * cl.cs));
+                cfg.blockDim = dim3(cl.nt);
+                cfg.dynamicSmemBytes = cl.smem;
+                cfg.stream = s;
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = cl.cs;
+                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                auto kern = cl.pg ? k_cluster_pcg<true, false, false>
+                            : cl.one ? (cl.ms ? k_cluster_pcg<false, true, true> : k_cluster_pcg<false, false, true>)
+                                     : (cl.ms ? k_cluster_pcg<false, true, false> : k_cluster_pcg<false, false, false>);
+                NVD_TRY_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
+                note_launch(1);
+            }
+        }
+        if (!direct) {
+            const int64_t nr = (int64_t)n_owner * kc;
+            k_cluster_collect<<<(unsigned)((nr + 127) / 128), 128, 0, s>>>(part, owners_dev, own, n_owner, kc, out + c0,
+                                                                           d2dev ? d2dev + c0 : nullptr);
+            note_launch(1);
+            NVD_TRY_CUDA(cudaGetLastError());
+        }
     }
     if (want_res) {
-        if (cst->h_cap < nres) {
-            if (cst->h_res) cudaFreeHost(cst->h_res);
-            cst->h_res = nullptr;
-            cst->h_cap = 0;
-            NVD_TRY_CUDA(cudaHostAlloc((void **)&cst->h_res, nres * sizeof(ColResult), cudaHostAllocDefault));
-            cst->h_cap = nres;
-        }
         NVD_TRY_CUDA(cudaMemcpyAsync(cst->h_res, out, nres * sizeof(ColResult), cudaMemcpyDeviceToHost, s));
         NVD_TRY_CUDA(cudaStreamSynchronize(s));
         *res = cst->h_res;

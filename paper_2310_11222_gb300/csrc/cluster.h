@@ -26,7 +26,8 @@ inline double tiles_iter_us(int64_t n, int64_t nnz, int kt, int tiles) {
 // Solve K columns for every owner (owners_dev: device table of n_owner, or NULL: own0);
 // the owners' x, y, z point at column 0 and hold kc columns.  d2dev: [K] device, one
 // owner only, or NULL.  want_res: read the [n_owner][K] results back (synchronises s)
-// into a buffer of the handle, valid until its next solve.
+// into a buffer of the handle, valid until its next solve.  NVD_ERR_OOM comes before anything
+// is launched.
 int cluster_solve(nvd_graph_s *g, ClusterPlan *pl, const nvd_solve_opts &o, const Owner *owners_dev, const Owner &own0,
                   int n_owner, int K, int xdt, bool write_z, double *d2dev, bool want_res, ColResult **res,
                   cudaStream_t s);

@@ -951,12 +951,26 @@ nvd_graph_s::~nvd_graph_s() {
 void *nvd_graph_s::wsp(const std::string &name, size_t bytes, int *st) {
     auto &slot = ws[name];
     if (!slot) slot.reset(new nvd::DevBuf());
-    int r = slot->ensure(bytes);
+    int r;
+    if (alloc_limit && bytes > alloc_limit && !(slot->p && bytes <= slot->bytes)) {
+        nvd::set_error("workspace of %zu bytes over the limit set for testing", bytes);
+        r = NVD_ERR_OOM;
+    } else {
+        r = slot->ensure(bytes);
+    }
     if (r != NVD_OK) {
         *st = r;
         return nullptr;
     }
     return slot->p;
+}
+
+void nvd_graph_s::drop_onchip() {
+    for (const char *name : {"cl_part", "cl_res", "cl_p", "rs_p", "rs_x", "rs_part", "rs_bar", "rs_res", "stage_x",
+                             "stage_y", "stage_z"})
+        ws.erase(name);
+    clusters.reset();
+    resident.reset();
 }
 
 int64_t nvd_graph_s::device_bytes() const {

@@ -162,9 +162,13 @@ struct nvd_graph_s {
     // (CTAs per cluster or columns per tile), and the form, width and kernel variant of the last one
     int32_t force_form = nvd::FORM_OPEN, force_width = 0;
     int32_t last_form = nvd::FORM_OPEN, last_width = 0, last_variant = 0;
+    size_t alloc_limit = 0;   // for the tests: larger workspaces find no memory (0: no limit)
     ~nvd_graph_s();
 
     void *wsp(const std::string &name, size_t bytes, int *st);
+    // Gives back the plans and workspaces of the on-chip solves (cluster.cu, resident.cu) and
+    // the staging they share with the tiles.
+    void drop_onchip();
     int64_t device_bytes() const;
 };
 
@@ -200,7 +204,11 @@ size_t l2_persist_bytes();
 // that graph took 121 ms.
 int target_blocks(const nvd_graph_s *g);
 // A status, with OK for "no memory": what is only a faster form is then left out.
-inline int unless_oom(int rc) { return rc == NVD_ERR_OOM ? (int)NVD_OK : rc; }
+inline int unless_oom(int rc) {
+    if (rc != NVD_ERR_OOM) return rc;
+    clear_error();
+    return NVD_OK;
+}
 // Fresh handle id.
 uint64_t next_graph_id();
 

@@ -87,5 +87,21 @@ inline int fill_onchip(const nvd_graph_s *g, int64_t n_tasks, int H, const FillT
     return NVD_OK;
 }
 
+// Pinned read-back buffer of at least n results.
+inline int pinned_results(ColResult **h, size_t *cap, size_t n) {
+    if (*cap >= n) return NVD_OK;
+    if (*h) cudaFreeHost(*h);
+    *h = nullptr;
+    *cap = 0;
+    if (cudaHostAlloc((void **)h, n * sizeof(ColResult), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        *h = nullptr;
+        set_error("no pinned memory for %zu results", n);
+        return NVD_ERR_OOM;
+    }
+    *cap = n;
+    return NVD_OK;
+}
+
 }  // namespace onchip
 }  // namespace nvd

@@ -723,6 +723,8 @@ int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, co
     unsigned *bar = (unsigned *)g->wsp("rs_bar", (size_t)(1 + ntiles) * 4, &st);
     ColResult *rd = (ColResult *)g->wsp("rs_res", (size_t)ntiles * KT * sizeof(ColResult), &st);
     if (st) return st;
+    const size_t need = (size_t)ntiles * KT + 1;
+    if (want_res) NVD_TRY(pinned_results(&rst->h_res, &rst->h_cap, need));   // the last thing that can lack memory
     NVD_TRY_CUDA(cudaMemsetAsync(bar, 0, (size_t)(1 + ntiles) * 4, s));
     for (int t = 0; t < ntiles; ++t) {
         const int c0 = t * KT, kc = std::min(KT, k - c0);
@@ -763,14 +765,6 @@ int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, co
         }
     }
     if (want_res) {
-        const size_t need = (size_t)ntiles * KT + 1;
-        if (rst->h_cap < need) {
-            if (rst->h_res) cudaFreeHost(rst->h_res);
-            rst->h_res = nullptr;
-            rst->h_cap = 0;
-            NVD_TRY_CUDA(cudaHostAlloc((void **)&rst->h_res, need * sizeof(ColResult), cudaHostAllocDefault));
-            rst->h_cap = need;
-        }
         int32_t *err = (int32_t *)(rst->h_res + (need - 1));
         NVD_TRY_CUDA(cudaMemcpyAsync(rst->h_res, rd, (need - 1) * sizeof(ColResult), cudaMemcpyDeviceToHost, s));
         NVD_TRY_CUDA(cudaMemcpyAsync(err, bar, 4, cudaMemcpyDeviceToHost, s));

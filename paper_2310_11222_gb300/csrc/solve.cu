@@ -89,8 +89,8 @@ int check_opts(const nvd_solve_opts &o) {
 // launch-by-launch profiling.  Three estimates of one iteration over all k columns decide:
 // one cluster per (component, pair) (cluster.cu), one persistent kernel with the vectors on
 // chip (resident.cu, the tile width of the least time), the host-driven tiles.  Host inputs
-// of the on-chip forms are staged whole, so only up to 256 MB of them.  A plan that finds no
-// memory leaves the solve to the tiles.
+// of the on-chip forms are staged whole, so only up to 256 MB of them.  A plan or workspace
+// that finds no memory leaves the solve to the tiles.
 int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size_t in_bytes, bool warm,
                 ClusterPlan **cluster, ResidentPlan **resident) {
     *cluster = nullptr;
@@ -212,7 +212,13 @@ int distance_impl(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_
         ClusterPlan *cpl = nullptr;
         ResidentPlan *rpl = nullptr;
         NVD_TRY(pick_onchip(g, o, k, KT, (size_t)k * g->n * (xdt == NVD_F64 ? 8 : 4), z0 != nullptr, &cpl, &rpl));
-        if (cpl || rpl) return onchip_distance(g, cpl, rpl, o, k, x, y, xdt, d2_out, z_out, stats, s, idx);
+        if (cpl || rpl) {
+            const int rc = onchip_distance(g, cpl, rpl, o, k, x, y, xdt, d2_out, z_out, stats, s, idx);
+            if (rc != NVD_ERR_OOM) return rc;
+            // nothing was launched: the tiles need less
+            clear_error();
+            g->drop_onchip();
+        }
     }
     g->last_form = FORM_TILES;
     g->last_width = KT;
@@ -948,5 +954,16 @@ extern "C" int nvd_diag_last_form(nvd_graph_t g, int32_t *form, int32_t *width, 
     *form = g->last_form;
     *width = g->last_width;
     *variant = g->last_variant;
+    return NVD_OK;
+}
+
+// For the package's tests: workspaces of more than `bytes` find no memory (0: no limit).
+extern "C" int nvd_diag_alloc_limit(nvd_graph_t g, int64_t bytes) {
+    clear_error();
+    if (!g || bytes < 0) {
+        set_error("nvd_diag_alloc_limit: invalid argument");
+        return NVD_ERR_INVALID_ARG;
+    }
+    g->alloc_limit = (size_t)bytes;
     return NVD_OK;
 }
