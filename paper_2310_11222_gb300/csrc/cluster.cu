@@ -504,9 +504,9 @@ struct ClClass {
 }  // namespace
 
 struct ClusterPlan {
-    int cs_max = 0;
+    bool fits = true;          // else nothing is on the device
     std::vector<ClClass> classes;
-    int64_t n_slots = 0, n_entries = 0;
+    int64_t n_slots = 0;
     DevBuf segs, ctas, items, col, w, node, deg, dinv;
     DevBuf tasks, slot_row, slot_of;   // what the weight updates need
     int64_t n_tasks = 0;
@@ -575,7 +575,6 @@ int cl_cs(int64_t n, int cs_max) {
 
 int build_cluster_plan(nvd_graph_s *g, int cs_max, ClusterPlan **out) {
     std::unique_ptr<ClusterPlan> pl(new ClusterPlan());
-    pl->cs_max = cs_max;
     const std::vector<int64_t> &rp = g->h_rowptr;
     const int nseg = g->nseg;
     std::vector<int32_t> owner(nseg, 0);
@@ -704,9 +703,13 @@ int build_cluster_plan(nvd_graph_s *g, int cs_max, ClusterPlan **out) {
         // publish p through L2 from 40 KB on (measured, barrier included: 2,080 clocks against
         // 2,350 at 18 KB, 4,160 against 3,450 at 65 KB, 15,300 against 5,800 at 164 KB)
         cl.l2 = cl.pg || (cl.cs > 1 && 8 * cl.max_slots > 40 * 1024);
+        pl->fits = pl->fits && cl.smem <= CL_SMEM_MAX;
+    }
+    if (!pl->fits) {
+        *out = pl.release();
+        return NVD_OK;
     }
     pl->n_slots = (int64_t)slot_row.size();
-    pl->n_entries = ne;
     auto up = [&](DevBuf &d, const void *h, size_t bytes) -> int {
         NVD_TRY(d.alloc(std::max<size_t>(bytes, 16)));
         if (bytes) NVD_TRY_CUDA(cudaMemcpy(d.p, h, bytes, cudaMemcpyHostToDevice));
@@ -848,9 +851,7 @@ int cluster_plan_get(nvd_graph_s *g, int cs, ClusterPlan **out) {
         }
         slot.reset(p);
     }
-    for (const ClClass &cl : slot->classes)
-        if (cl.smem > CL_SMEM_MAX) return NVD_OK;
-    *out = slot.get();
+    if (slot->fits) *out = slot.get();
     return NVD_OK;
 }
 
@@ -862,7 +863,8 @@ void cluster_variant(const ClusterPlan *pl, int32_t *cs, int32_t *variant) {
 
 int cluster_refill(nvd_graph_s *g, cudaStream_t s) {
     if (!g->clusters) return NVD_OK;
-    for (auto &kv : g->clusters->plans) NVD_TRY(fill_cluster_plan(g, kv.second.get(), s));
+    for (auto &kv : g->clusters->plans)
+        if (kv.second->fits) NVD_TRY(fill_cluster_plan(g, kv.second.get(), s));
     return NVD_OK;
 }
 

@@ -112,25 +112,30 @@ int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size
         set_error("the form asked for does not fit the graph");
         return NVD_ERR_UNSUPPORTED;
     }
-    double best = tiles_iter_us(g->n, g->nnz, KT, (k + KT - 1) / KT), us = 0.0;
-    int cs = 0, rkt = 0;
-    NVD_TRY(cluster_estimate(g, k, &cs, &us));
-    if (cs && us < best) best = us;
-    else cs = 0;
+    // every estimate before the first plan: building one takes longer than most solves
+    struct Form {
+        double us;
+        int kt, cs;   // columns per tile (one kernel) or CTAs per cluster
+    };
+    std::vector<Form> forms;
+    Form c{0.0, 0, 0};
+    NVD_TRY(cluster_estimate(g, k, &c.cs, &c.us));
+    if (c.cs) forms.push_back(c);
     // a call without a final synchronisation has nobody to report a wait that gave up to
     if (g->nseg == 1 && !(o.flags & NVD_SOLVE_NO_SYNC))
         for (int kt : {1, 4, 8, 16}) {
             if (kt > KT && kt > 1) break;
-            us = ((k + kt - 1) / kt) * resident_iter_us(g->h_seg_end[0] - g->h_seg_begin[0], g->nnz, kt);
-            ResidentPlan *pl = nullptr;
-            if (us < best) NVD_TRY(unless_oom(resident_plan_for(g, kt, &pl)));
-            if (pl) {
-                best = us;
-                rkt = kt;
-                *resident = pl;
-            }
+            forms.push_back(Form{((k + kt - 1) / kt) * resident_iter_us(g->h_seg_end[0] - g->h_seg_begin[0], g->nnz, kt),
+                                 kt, 0});
         }
-    if (!rkt && cs) NVD_TRY(unless_oom(cluster_plan_get(g, cs, cluster)));
+    std::stable_sort(forms.begin(), forms.end(), [](const Form &u, const Form &v) { return u.us < v.us; });
+    const double tiles = tiles_iter_us(g->n, g->nnz, KT, (k + KT - 1) / KT);
+    for (const Form &f : forms) {
+        if (!(f.us < tiles)) break;
+        if (f.cs) NVD_TRY(unless_oom(cluster_plan_get(g, f.cs, cluster)));
+        else NVD_TRY(unless_oom(resident_plan_for(g, f.kt, resident)));
+        if (*cluster || *resident) break;
+    }
     return NVD_OK;
 }
 

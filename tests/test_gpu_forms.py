@@ -183,3 +183,39 @@ def test_one_kernel_wait_that_gives_up(nvd, case):
     force(nvd, G, 0, 0)
     t = nvd.ge_distance(G, on(X), on(Y), rtol=1e-11, test_timeout=True).cpu().numpy()
     assert last(nvd, G)[0] == TILES and rel(t, want) < 1e-10
+
+
+# 5 pairs: tiles of 4 and of 8 columns are both estimated to beat the host-driven ones; 16 pairs: 8 and 16
+@pytest.mark.parametrize("n,k", [(100003, 5), (70001, 16), (31003, 16), (2000, 16)])
+def test_only_the_plan_that_is_used_is_built(nvd, n, k):
+    rng = np.random.default_rng(n)
+    eu, ev = synth.watts_strogatz(n, 10, 0.3, rng)
+    g = synth.csr_from_edges(n, eu, ev, rng.uniform(0.5, 2.0, len(eu)))
+    x, y = torch.rand(k, n, dtype=torch.float64, device=DEV), torch.rand(k, n, dtype=torch.float64, device=DEV)
+    G = nvd.Graph.from_csr(g)
+    d2 = nvd.ge_distance(G, x, y, rtol=1e-10)
+    form, width, _ = last(nvd, G)
+    H = nvd.Graph.from_csr(g)
+    force(nvd, H, form, 16 if form == CLUSTER else width)
+    assert torch.equal(d2, nvd.ge_distance(H, x, y, rtol=1e-10))
+    assert last(nvd, H)[:2] == (form, width)
+    assert G.info()["device_bytes"] == H.info()["device_bytes"]
+
+
+def test_a_cluster_plan_that_does_not_fit_holds_no_memory(nvd):
+    """Hubs take so much of some CTAs' time that the others' rows exceed their shared memory: the
+    form is refused when asked for, and an open call takes another."""
+    n = 100000
+    g = hub_graph(n, [60000] * 8, 4)
+    X, Y = synth.sparse_uniform_pairs(g.n, 3, 0.02, 5)
+    G = nvd.Graph.from_csr(g)
+    before = G.info()["device_bytes"]
+    force(nvd, G, CLUSTER, 16)
+    with pytest.raises(nvd.NvdError) as e:
+        nvd.ge_distance(G, on(X), on(Y), rtol=1e-11)
+    assert e.value.status == 9 and G.info()["device_bytes"] == before
+    G.set_weights(g.w)
+    force(nvd, G, 0, 0)
+    d2 = nvd.ge_distance(G, on(X), on(Y), rtol=1e-11).cpu().numpy()
+    assert last(nvd, G)[0] != CLUSTER
+    assert rel(d2, ocg.ge_d2_cg(g.n, g.rowptr, g.colidx, g.w, X, Y, rtol=1e-13)[0]) < 1e-10
