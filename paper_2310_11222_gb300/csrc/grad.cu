@@ -11,7 +11,8 @@
 // The weight gradient is a gather over the undirected edges: z is first laid out as
 // [n][KT] tiles (one 16-byte aligned row per node); an edge reads its two nodes' rows and
 // writes its two stored entries, which have the same derivative.  The edge list (its nodes
-// and the places of its entries) is made from the CSR once per handle.
+// and the places of its entries) is made from the CSR once per handle; without memory for it
+// the stored entries are taken one by one.
 #include <algorithm>
 #include <cstring>
 #include <utility>
@@ -179,6 +180,42 @@ __global__ void __launch_bounds__(256) k_grad_edges(int64_t n_edges, const int2 
     }
 }
 
+// The same without the edge list (24 bytes per edge), for a handle that has no memory for it:
+// one warp per row, a lane group per stored entry.
+template <class TZ, class TG, int KT, bool ACC>
+__global__ void __launch_bounds__(256) k_grad_rows(int64_t n, const int64_t *__restrict__ rowptr,
+                                                   const int32_t *__restrict__ colidx, const TZ *__restrict__ zt,
+                                                   const double *__restrict__ gb, TG *__restrict__ g) {
+    constexpr int VEC = dev::VecCfg<TZ, KT>::VEC, LPR = KT / VEC, G = 32 / LPR;
+    const int lane = threadIdx.x & 31, gi = lane / LPR, col0 = (lane % LPR) * VEC;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
+        const int64_t e1 = __ldg(rowptr + u + 1);
+        TZ own[VEC];
+        dev::ldv<dev::LdRO, TZ, VEC>(zt + u * KT + col0, own);
+        for (int64_t eb = __ldg(rowptr + u); eb < e1; eb += G) {
+            const int64_t e = eb + gi;
+            double s = 0.0;
+            if (e < e1) {
+                TZ zv[VEC];
+                dev::ldv<dev::LdRO, TZ, VEC>(zt + (int64_t)__ldcs(colidx + e) * KT + col0, zv);
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) {
+                    const double d = to_f64(own[q]) - to_f64(zv[q]);
+                    s += __ldg(gb + col0 + q) * d * d;
+                }
+            }
+#pragma unroll
+            for (int off = 1; off < LPR; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            if (e < e1 && col0 == 0) {
+                const double val = -0.5 * s;
+                if (ACC) g[e] = (TG)((double)g[e] + val);
+                else g[e] = (TG)val;
+            }
+        }
+    }
+}
+
 // grad_w[e] = g_int[uent[e]] (0 for dropped self-loops), converted to TW.
 template <class TW>
 __global__ void k_grad_scatter(const double *__restrict__ gint, const int64_t *__restrict__ uent,
@@ -231,8 +268,8 @@ int edge_list(nvd_graph_s *g, cudaStream_t s) {
     unsigned long long ne = 0, written = 0;
     NVD_TRY(run(k_edge_list<false>, nullptr, nullptr, &ne));
     DevBuf uv, at;
-    NVD_TRY(uv.alloc((size_t)ne * sizeof(int2)));
-    NVD_TRY(at.alloc((size_t)ne * sizeof(longlong2)));
+    NVD_TRY(g->grow(uv, (size_t)ne * sizeof(int2)));
+    NVD_TRY(g->grow(at, (size_t)ne * sizeof(longlong2)));
     NVD_TRY(run(k_edge_list<true>, uv.as<int2>(), at.as<longlong2>(), &written));
     std::swap(g->grad_uv.p, uv.p);
     std::swap(g->grad_uv.bytes, uv.bytes);
@@ -258,19 +295,27 @@ int grad_w_impl(nvd_graph_s *g, int k, const TZ *z, const double *gbar, TW *grad
         if (st) return st;
     }
     const int zgrid = (int)((g->n + 31) / 32);
-    NVD_TRY(edge_list(g, s));
+    NVD_TRY(unless_oom(edge_list(g, s)));
+    const bool list = g->grad_uv.p != nullptr;
     const int64_t ne = g->grad_edges;
     const int2 *uv = g->grad_uv.as<int2>();
     const longlong2 *at = g->grad_at.as<longlong2>();
-    const int egrid = grid_cap(ne * (KT >= 8 ? 2 : 1), g->num_sms);
+    const int64_t *rp = g->rowptr.as<int64_t>();
+    const int32_t *ci = g->colidx.as<int32_t>();
+    const int egrid = grid_cap(list ? ne * (KT >= 8 ? 2 : 1) : g->n * 32, g->num_sms);
     for (int t = 0; t < ntile; ++t) {
+        const double *gbt = gbp + t * KT;
         k_z_tile<TZ, KT><<<zgrid, 256, 0, s>>>(z, g->n, k, t * KT, g->perm.as<int32_t>(), zt);
-        if (direct)
-            k_grad_edges<TZ, TW, KT, false><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbp, grad_w);
-        else if (t == 0)
-            k_grad_edges<TZ, double, KT, false><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbp, gint);
-        else
-            k_grad_edges<TZ, double, KT, true><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbp + t * KT, gint);
+        if (direct) {
+            if (list) k_grad_edges<TZ, TW, KT, false><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbt, grad_w);
+            else k_grad_rows<TZ, TW, KT, false><<<egrid, 256, 0, s>>>(g->n, rp, ci, zt, gbt, grad_w);
+        } else if (t == 0) {
+            if (list) k_grad_edges<TZ, double, KT, false><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbt, gint);
+            else k_grad_rows<TZ, double, KT, false><<<egrid, 256, 0, s>>>(g->n, rp, ci, zt, gbt, gint);
+        } else {
+            if (list) k_grad_edges<TZ, double, KT, true><<<egrid, 256, 0, s>>>(ne, uv, at, zt, gbt, gint);
+            else k_grad_rows<TZ, double, KT, true><<<egrid, 256, 0, s>>>(g->n, rp, ci, zt, gbt, gint);
+        }
         NVD_TRY_CUDA(cudaGetLastError());
     }
     if (!direct) {

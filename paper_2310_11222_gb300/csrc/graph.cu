@@ -948,16 +948,18 @@ nvd_graph_s::~nvd_graph_s() {
     if (copy_stream) cudaStreamDestroy(copy_stream);
 }
 
+int nvd_graph_s::grow(nvd::DevBuf &d, size_t bytes) {
+    if (alloc_limit && bytes > alloc_limit && !(d.p && bytes <= d.bytes)) {
+        nvd::set_error("%zu bytes are over the limit set for testing", bytes);
+        return NVD_ERR_OOM;
+    }
+    return d.ensure(bytes);
+}
+
 void *nvd_graph_s::wsp(const std::string &name, size_t bytes, int *st) {
     auto &slot = ws[name];
     if (!slot) slot.reset(new nvd::DevBuf());
-    int r;
-    if (alloc_limit && bytes > alloc_limit && !(slot->p && bytes <= slot->bytes)) {
-        nvd::set_error("workspace of %zu bytes over the limit set for testing", bytes);
-        r = NVD_ERR_OOM;
-    } else {
-        r = slot->ensure(bytes);
-    }
+    const int r = grow(*slot, bytes);
     if (r != NVD_OK) {
         *st = r;
         return nullptr;

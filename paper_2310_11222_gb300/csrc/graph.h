@@ -166,6 +166,7 @@ struct nvd_graph_s {
     ~nvd_graph_s();
 
     void *wsp(const std::string &name, size_t bytes, int *st);
+    int grow(nvd::DevBuf &d, size_t bytes);   // to at least that many
     // Gives back the plans and workspaces of the on-chip solves (cluster.cu, resident.cu) and
     // the staging they share with the tiles.
     void drop_onchip();

@@ -143,3 +143,34 @@ def test_batches_without_memory(nvd):
     want = np.concatenate([ocg.ge_d2_cg(g.n, g.rowptr, g.colidx, g.w, x, y, rtol=1e-13)[0]
                            for g, (x, y) in zip(gs, pairs)])
     assert rel(d2, want) < 1e-10 and rel(d2c, want) < 1e-10
+
+
+# One direction of every pair only: the 130,816 entries are an edge each, 16 bytes of places and 8
+# of nodes.  z tile 512 nodes x 32 columns x 8 bytes = 131 KB; with several tiles or unsorted columns
+# the gradient of every entry, 8 bytes (1,046,528 in all).
+@pytest.mark.parametrize("k", [1, 4, 7, 16, 32, 40])
+@pytest.mark.parametrize("zt,wt", [(np.float64, np.float64), (np.float32, np.float32), (np.float64, np.float32)])
+def test_weight_gradient_without_an_edge_list(nvd, k, zt, wt):
+    rng = np.random.default_rng([k, 4])
+    n = 512
+    rows, cols = np.triu_indices(n, 1)
+    rowptr = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=n))])
+    if k >= 16:                                  # unsorted columns: entries reach the handle by a map
+        cols[[0, 1]] = cols[[1, 0]]
+    G = nvd.Graph(rowptr, cols.astype(np.int32), np.ones(len(rows), wt), skip_sym_check=True)
+    z = rng.standard_normal((k, n)).astype(zt)
+    gbar = rng.uniform(-1.0, 1.0, k)
+    args = (torch.as_tensor(z, device=DEV), torch.as_tensor(gbar, device=DEV))
+    limit(nvd, G, 1100000)
+    before = G.info()["device_bytes"]
+    gw = nvd.ge_grad(G, *args)[0].cpu().numpy()
+    assert G.info()["device_bytes"] - before < 1300000
+    d = z.astype(np.float64)[:, rows] - z.astype(np.float64)[:, cols]
+    want, size = -0.5 * (gbar[:, None] * d * d).sum(0), 0.5 * (np.abs(gbar)[:, None] * d * d).sum(0)
+    # FP64 sums of k terms; rounded once to the weights' type
+    tol = 1e-13 * size + (1e-7 * np.abs(want) if wt == np.float32 else 0.0)
+    assert np.all(np.abs(gw - want) <= tol + 1e-300)
+    limit(nvd, G, 0)
+    full = nvd.ge_grad(G, *args)[0].cpu().numpy()
+    assert G.info()["device_bytes"] - before > 3000000
+    assert np.all(np.abs(full - want) <= tol + 1e-300)
