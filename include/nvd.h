@@ -196,7 +196,9 @@ typedef struct {
     int32_t row_max_pct;   /* light-row limit in percent of the default (50, 100 or 200) */
     int32_t blocks_pct;    /* light CTA blocks per SpMV in percent of the default, one wave of four
                               per SM (below 100: as 100) */
-    int32_t persistent;    /* 1: one persistent launch per tile was faster */
+    int32_t persistent;    /* 1: one persistent launch per tile was faster; -1 (only with
+                              NVD_TUNE_SINGLE_RHS in FP64): host-driven launches were faster than
+                              the one-launch form that an open call would take */
     int32_t candidates;    /* configurations timed */
     int32_t fold_direction; /* 1: two kernels per iteration (NVD_SOLVE_FOLD_DIRECTION) were faster */
     int32_t gather;        /* multi-column SpMM: 0 register loads per slice (default), 1 register loads
@@ -226,8 +228,10 @@ typedef struct {
  * when opts.kt = 0 and the launch mode and iteration form when the flags leave
  * them at their defaults.
  * With NVD_TUNE_SINGLE_RHS in FP64 mode the form an open call takes by itself is
- * timed too; otherwise a tuned FP64 handle keeps its tiles, and a graph that fits
- * the one-launch forms (nvd_ge_distance) is better left untuned.
+ * timed too, and the result, here or through nvd_graph_set_tuning, says which of
+ * the two later calls of one right-hand side at a time take; otherwise a tuned
+ * FP64 handle keeps its tiles, and a graph that fits the one-launch forms
+ * (nvd_ge_distance) is better left untuned.
  * Results do not depend on the choice beyond rounding (each choice is a valid
  * order of the same sums).  Synchronous.
  *   k      number of pairs the later calls will solve (sets the tile-width cost
@@ -244,8 +248,9 @@ int nvd_graph_tune(nvd_graph_t g, int32_t mode, int32_t k, uint32_t flags, nvd_t
 /*
  * nvd_graph_set_tuning -- apply a setting (for example one nvd_graph_tune chose
  * earlier for the same graph) without timing anything.  Reads kt (0 = no
- * preference), row_max_pct and blocks_pct (10..1000), persistent,
- * fold_direction and l2_hot (0/1), gather (0..3); the other fields are ignored.  Host only; plans built
+ * preference), row_max_pct and blocks_pct (10..1000), persistent
+ * (-1, 0 or 1), fold_direction and l2_hot (0/1), gather (0..3); the other fields are
+ * ignored.  Host only; plans built
  * afterwards use it.
  * Errors: NVD_ERR_INVALID_ARG (NULL pointer, bad mode or field).
  */
@@ -268,8 +273,8 @@ int nvd_graph_set_tuning(nvd_graph_t g, int32_t mode, const nvd_tune_result *t);
  * returns NVD_ERR_NOT_CONVERGED; per-pair status is in stats.
  *
  * An FP64 solve that leaves its form open (opts kt = 0, no NVD_SOLVE_PERSISTENT,
- * FOLD_DIRECTION or TEST_TIMEOUT, no tile width or such form chosen by
- * nvd_graph_tune) runs as one thread-block cluster per (component, pair), as one cooperative kernel with the
+ * FOLD_DIRECTION or TEST_TIMEOUT, no tile width above 1 or such form chosen by
+ * nvd_graph_tune, a width of 1 only for one right-hand side at a time) runs as one thread-block cluster per (component, pair), as one cooperative kernel with the
  * vectors in shared memory (one component, not with NVD_SOLVE_NO_SYNC), or as
  * host-driven launches over tiles of columns, whichever is estimated to take the
  * least time on this graph; the stopping rule is the same in all three.  Where the first two

@@ -327,14 +327,16 @@ class Graph:
         return {f: getattr(r, f) for f, _ in TuneResult._fields_}
 
     def set_tuning(self, *, mode: int = 0, kt: int = 0, row_max_pct: int = 100, blocks_pct: int = 100,
-                   persistent: bool = False, fold_direction: bool = False, gather: int = GATHER_SLICES,
+                   persistent: int = False, fold_direction: bool = False, gather: int = GATHER_SLICES,
                    l2_hot: bool = False):
-        """Apply a work-decomposition setting without timing (``nvd_graph_set_tuning``).
+        """Apply a work-decomposition setting without timing (``nvd_graph_set_tuning``), for
+        example fields of an earlier ``tune`` result (``persistent`` may be -1 there).
         ``gather``: GATHER_SLICES (default), GATHER_STREAM, GATHER_TMA or GATHER_ACOPY; ``l2_hot``: keep the
         highest-degree rows of a degree-ordered graph persisting in L2."""
         r = TuneResult(kt=int(kt), row_max_pct=int(row_max_pct), blocks_pct=int(blocks_pct),
-                       persistent=int(bool(persistent)), fold_direction=int(bool(fold_direction)),
-                       gather=int(gather), l2_hot=int(bool(l2_hot)))
+                       persistent=-1 if persistent == -1 else int(bool(persistent)),
+                       fold_direction=int(bool(fold_direction)), gather=int(gather),
+                       l2_hot=int(bool(l2_hot)))
         _check(self._lib.nvd_graph_set_tuning(self.handle, int(mode), ctypes.byref(r)), "nvd_graph_set_tuning")
 
     @property

@@ -140,7 +140,9 @@ struct nvd_graph_s {
     nvd::DevBuf seg_begin, seg_end, seg_owner;
     nvd::SpParams sp;            // parameters of plans built from now on (nvd_graph_tune)
     int32_t tuned_kt[3] = {0, 0, 0};          // per solve mode: tile width chosen by the tuner (0 = none)
-    int32_t tuned_persistent[3] = {0, 0, 0};  // per solve mode: 1 = persistent launch was faster
+    // per solve mode: 1 = persistent launch was faster; -1 = for single right-hand sides in FP64
+    // the tiles were faster than the on-chip form an open call would take
+    int32_t tuned_persistent[3] = {0, 0, 0};
     int32_t tuned_fold[3] = {0, 0, 0};        // per solve mode: 1 = two kernels per iteration were faster
     std::map<int64_t, std::unique_ptr<nvd::Plan>> plans;
     std::map<std::string, std::unique_ptr<nvd::DevBuf>> ws;  // named lazily-grown workspace

@@ -85,7 +85,7 @@ int check_opts(const nvd_solve_opts &o) {
 }
 
 // Which form an FP64 solve takes when the call leaves it open: no tile width, persistent or
-// folded form, here or from the tuner (which times tiles), a start from zero and no
+// folded form, here or from the tuner (nor, for single right-hand sides, tiles it found faster), a start from zero and no
 // launch-by-launch profiling.  Three estimates of one iteration over all k columns decide:
 // one cluster per (component, pair) (cluster.cu), one persistent kernel with the vectors on
 // chip (resident.cu, the tile width of the least time), the host-driven tiles.  Host inputs
@@ -95,8 +95,10 @@ int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size
                 ClusterPlan **cluster, ResidentPlan **resident) {
     *cluster = nullptr;
     *resident = nullptr;
-    if (o.mode != NVD_MODE_FP64 || o.kt || warm || prof_enabled() || g->tuned_kt[o.mode] ||
-        g->tuned_persistent[o.mode] || g->tuned_fold[o.mode] ||
+    // one right-hand side at a time has no width to choose: a tuned width of 1 leaves the form open
+    const bool single = k == 1 || (o.flags & NVD_SOLVE_SINGLE_RHS);
+    if (o.mode != NVD_MODE_FP64 || o.kt || warm || prof_enabled() || g->tuned_kt[o.mode] > (single ? 1 : 0) ||
+        g->tuned_persistent[o.mode] > 0 || (single && g->tuned_persistent[o.mode] < 0) || g->tuned_fold[o.mode] ||
         (o.flags & (NVD_SOLVE_PERSISTENT | NVD_SOLVE_FOLD_DIRECTION)) ||
         // (the timeout test reaches only the form with a grid barrier, and that only when forced)
         ((o.flags & NVD_SOLVE_TEST_TIMEOUT) && g->force_form != FORM_RESIDENT) ||
@@ -235,7 +237,7 @@ int distance_impl(nvd_graph_t g, int32_t k, const void *x, const void *y, int32_
     const bool d2_dev = o.flags & NVD_SOLVE_D2_DEVICE;
     // persistent single-launch solve (FP64/FP32 modes; the launch timer needs the host
     // loop); it runs the register-path SpMM, so it takes a plan laid out for that
-    const bool persistent = ((o.flags & NVD_SOLVE_PERSISTENT) || g->tuned_persistent[o.mode]) && !mixed &&
+    const bool persistent = ((o.flags & NVD_SOLVE_PERSISTENT) || g->tuned_persistent[o.mode] > 0) && !mixed &&
                             !prof_enabled() && !z0;
     Plan *pl = nullptr, *pl64 = nullptr;
     NVD_TRY(get_plan(g, KT, (int)szv, (int)szv, &pl, !persistent));

@@ -309,7 +309,9 @@ int tune_impl(nvd_graph_s *g, int32_t mode, int32_t k, uint32_t flags, nvd_tune_
     // 6. single right-hand sides in FP64: the form an open call takes by itself (one launch
     //    with the vectors on chip where that is estimated to be faster), all of them in one
     //    call, against the best tile one after the other.  One pair on 1,000..10^5 nodes of
-    //    mean degree 8, whole call: ER 0.60 to 0.19, 0.66 to 0.31, 0.90 to 0.46 ms.
+    //    mean degree 8, whole call: ER 0.60 to 0.19, 0.66 to 0.31, 0.90 to 0.46 ms.  The host-driven
+    //    tiles are recorded as such (persistent -1) where they win, or later open calls would take
+    //    the other form by its estimate.
     if (single && mode == NVD_MODE_FP64) {
         const int cols = std::min(k, 32);
         double it = INFINITY;
@@ -321,6 +323,8 @@ int tune_impl(nvd_graph_s *g, int32_t mode, int32_t k, uint32_t flags, nvd_tune_
         if (it < cols * best_iter * 0.97) {
             pers = fold = 0;
             best_iter = it / cols;
+        } else if (!pers && !fold && it > cols * best_iter * 1.03) {
+            pers = -1;
         }
     }
     restore_timed();
@@ -356,7 +360,7 @@ extern "C" int nvd_graph_set_tuning(nvd_graph_t g, int32_t mode, const nvd_tune_
     if (!g || !t || mode < NVD_MODE_FP64 || mode > NVD_MODE_MIXED ||
         !(t->kt == 0 || t->kt == 1 || t->kt == 4 || t->kt == 8 || t->kt == 16 || t->kt == 32) ||
         t->row_max_pct < 10 || t->row_max_pct > 1000 || t->blocks_pct < 10 || t->blocks_pct > 1000 ||
-        (t->persistent != 0 && t->persistent != 1) || (t->fold_direction != 0 && t->fold_direction != 1) ||
+        t->persistent < -1 || t->persistent > 1 || (t->fold_direction != 0 && t->fold_direction != 1) ||
         t->gather < 0 || t->gather > 3 || (t->l2_hot != 0 && t->l2_hot != 1)) {
         set_error("nvd_graph_set_tuning: invalid argument");
         return NVD_ERR_INVALID_ARG;
