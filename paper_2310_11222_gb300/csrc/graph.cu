@@ -605,8 +605,9 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
     const int gm = (!allow_stream || KT == 1 || g->sp.gather <= 0) ? 0
                    : (g->sp.gather >= 2 && tma_tile(KT, szv)) ? std::min(g->sp.gather, 3) : 1;
     const bool tma = gm != 0;   // stream layout (the name of the TMA plans it began with)
+    const int32_t blocks_pct = std::max(g->sp.blocks_pct, 100);   // a smaller value is the same plan
     const int64_t key = ((int64_t)(KT * 256 + szv * 16 + sza) << 32) | ((int64_t)gm << 30) |
-                        ((int64_t)g->sp.row_max_pct << 16) | (int64_t)g->sp.blocks_pct;
+                        ((int64_t)g->sp.row_max_pct << 16) | (int64_t)blocks_pct;
     auto it = g->plans.find(key);
     if (it != g->plans.end()) {
         *out = it->second.get();
@@ -617,6 +618,7 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
     pl->szv = szv;
     pl->sza = sza;
     pl->sp = g->sp;
+    pl->sp.blocks_pct = blocks_pct;
     const int64_t RMAX = std::max<int64_t>(
         1, (int64_t)(tma ? sp_row_max_stream(KT, szv) : sp_row_max(KT, szv)) * g->sp.row_max_pct / 100);
     const int64_t LONG = sp_long_max(KT);
@@ -699,7 +701,7 @@ int get_plan(nvd_graph_s *g, int KT, int szv, int sza, Plan **out, bool allow_st
         heavy_blocks = 0;
         if (!tma) waves = (int)std::min<int64_t>(4, std::max<int64_t>(1, seg_rows * KT * szv / 22000000));
     }
-    const int wave = waves * target_blocks(g) * std::max(g->sp.blocks_pct, 100) / 100;
+    const int wave = waves * target_blocks(g) * blocks_pct / 100;
     const int T = std::max<int>(1, wave - (heavy_blocks <= wave / 4 ? (int)std::min<int64_t>(heavy_blocks, wave / 10) : 0));
     const double target = ltot / T;
     // block sizes in whole slices (warps take a block's slices as they free up)
