@@ -144,7 +144,9 @@ struct Ctx {
     // ---- sliced copy of the light rows: slice s holds H = sp_slice_rows rows
     //      sl_row[s*H + r] (-1 = empty lane group); entry j of row r sits at
     //      sl_base[s] + j*H + r of sl_col / sl_w (TW); rows shorter than the slice's
-    //      longest are padded with zero weights on their own column
+    //      longest are padded with zero weights on their own column.  A slice of one long
+    //      row (sp_group_max) has its id at r = 0 and -2 elsewhere, and its entry e at
+    //      sl_base[s] + e
     const int64_t *sl_base;         // [n_slices + 1]
     const int32_t *sl_row;          // [n_slices * H]
     const int32_t *sl_col;

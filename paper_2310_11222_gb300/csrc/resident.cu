@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
             if (valid && (!finite(rr) || !finite(rho))) st.status[c] = NVD_ERR_NUMERIC;
             const int act = valid && pos_finite(rr) && pos_finite(rho);
             st.active[c] = act;
-            const unsigned all = KT == 32 ? 0xffffffffu : (1u << KT) - 1u;
+            const unsigned all = (1u << KT) - 1u;
             const unsigned any = __ballot_sync(all, act);
             if (c == 0) st.go = any != 0;
         }, nothing)))
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
                         st.rho[c] = rho_new;
                     }
                 }
-                const unsigned all = KT == 32 ? 0xffffffffu : (1u << KT) - 1u;
+                const unsigned all = (1u << KT) - 1u;
                 const unsigned any = __ballot_sync(all, act);
                 if (c == 0) st.go = any != 0;
             },
@@ -710,7 +710,7 @@ int resident_refill(nvd_graph_s *g, cudaStream_t s) {
 }
 
 int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, const Owner &own, int k, int xdt,
-                   double *d2dev, bool want_res, ColResult **res, cudaStream_t s) {
+                   double *d2dev, ColResult **res, cudaStream_t s) {
     ResidentState *rst = g->resident.get();
     const int KT = pl->KT, ntiles = (k + KT - 1) / KT;
     const size_t xsz = own.idx ? 4 : xdt == NVD_F64 ? 8 : 4, zsz = xdt == NVD_F64 ? 8 : 4;
@@ -724,7 +724,7 @@ int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, co
     ColResult *rd = (ColResult *)g->wsp("rs_res", (size_t)ntiles * KT * sizeof(ColResult), &st);
     if (st) return st;
     const size_t need = (size_t)ntiles * KT + 1;
-    if (want_res) NVD_TRY(pinned_results(&rst->h_res, &rst->h_cap, need));   // the last thing that can lack memory
+    NVD_TRY(pinned_results(&rst->h_res, &rst->h_cap, need));   // the last thing that can lack memory
     NVD_TRY_CUDA(cudaMemsetAsync(bar, 0, (size_t)(1 + ntiles) * 4, s));
     for (int t = 0; t < ntiles; ++t) {
         const int c0 = t * KT, kc = std::min(KT, k - c0);
@@ -764,17 +764,15 @@ int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, co
             default: NVD_TRY(launch<16>(pl, a, s)); break;
         }
     }
-    if (want_res) {
-        int32_t *err = (int32_t *)(rst->h_res + (need - 1));
-        NVD_TRY_CUDA(cudaMemcpyAsync(rst->h_res, rd, (need - 1) * sizeof(ColResult), cudaMemcpyDeviceToHost, s));
-        NVD_TRY_CUDA(cudaMemcpyAsync(err, bar, 4, cudaMemcpyDeviceToHost, s));
-        NVD_TRY_CUDA(cudaStreamSynchronize(s));
-        if (*err) {
-            set_error("nvd_ge_distance: a bounded device wait gave up (status %d)", *err);
-            return *err;
-        }
-        *res = rst->h_res;
+    int32_t *err = (int32_t *)(rst->h_res + (need - 1));
+    NVD_TRY_CUDA(cudaMemcpyAsync(rst->h_res, rd, (need - 1) * sizeof(ColResult), cudaMemcpyDeviceToHost, s));
+    NVD_TRY_CUDA(cudaMemcpyAsync(err, bar, 4, cudaMemcpyDeviceToHost, s));
+    NVD_TRY_CUDA(cudaStreamSynchronize(s));
+    if (*err) {
+        set_error("nvd_ge_distance: a bounded device wait gave up (status %d)", *err);
+        return *err;
     }
+    *res = rst->h_res;
     return NVD_OK;
 }
 

@@ -19,11 +19,11 @@ int32_t resident_width(const ResidentPlan *pl);
 int32_t resident_variant(const ResidentPlan *pl);
 
 // Solve k columns, tile after tile (own: x, y, z at column 0).  d2dev: [k] device or NULL.
-// want_res: read the [k] results back (synchronises s) into a buffer of the handle, valid
-// until its next solve; without it a bounded wait that gave up goes unreported.  NVD_ERR_OOM
+// Synchronises s and reads the [k] results back into a buffer of the handle, valid until its
+// next solve: a bounded wait that gave up is reported by this call or not at all.  NVD_ERR_OOM
 // comes before anything is launched.
 int resident_solve(nvd_graph_s *g, ResidentPlan *pl, const nvd_solve_opts &o, const Owner &own, int k, int xdt,
-                   double *d2dev, bool want_res, ColResult **res, cudaStream_t s);
+                   double *d2dev, ColResult **res, cudaStream_t s);
 
 // New weights in the cached plans (nvd_graph_set_weights).
 int resident_refill(nvd_graph_s *g, cudaStream_t s);

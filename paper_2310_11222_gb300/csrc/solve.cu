@@ -147,7 +147,6 @@ int onchip_distance(nvd_graph_t g, ClusterPlan *cpl, ResidentPlan *rpl, const nv
     const size_t xsz = xdt == NVD_F64 ? 8 : 4, bytes = (size_t)k * g->n * xsz;
     const bool host_in = o.flags & NVD_SOLVE_HOST_INPUTS, d2_dev = o.flags & NVD_SOLVE_D2_DEVICE;
     const bool report = !d2_dev || stats || host_in;   // per-pair results go back to the caller
-    const bool want = report || rpl;
     int st = NVD_OK;
     void *z = z_out;
     double *d2 = d2_dev ? d2_out : nullptr;
@@ -170,10 +169,10 @@ int onchip_distance(nvd_graph_t g, ClusterPlan *cpl, ResidentPlan *rpl, const nv
         cluster_variant(cpl, &g->last_width, &g->last_variant);
     }
     ColResult *res = nullptr;
-    if (rpl) NVD_TRY(resident_solve(g, rpl, o, own, k, xdt, d2, want, &res, s));
-    else NVD_TRY(cluster_solve(g, cpl, o, nullptr, own, 1, k, xdt, z != nullptr, d2, want, &res, s));
+    if (rpl) NVD_TRY(resident_solve(g, rpl, o, own, k, xdt, d2, &res, s));
+    else NVD_TRY(cluster_solve(g, cpl, o, nullptr, own, 1, k, xdt, z != nullptr, d2, report, &res, s));
     if (host_in && z_out) NVD_TRY_CUDA(cudaMemcpyAsync(z_out, z, bytes, cudaMemcpyDeviceToHost, s));
-    if (!(o.flags & NVD_SOLVE_NO_SYNC) || want) NVD_TRY_CUDA(cudaStreamSynchronize(s));
+    if (!(o.flags & NVD_SOLVE_NO_SYNC) || report) NVD_TRY_CUDA(cudaStreamSynchronize(s));
     int overall = NVD_OK;
     if (report)
         for (int32_t j = 0; j < k; ++j) {
