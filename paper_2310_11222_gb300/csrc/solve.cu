@@ -119,21 +119,25 @@ int pick_onchip(nvd_graph_s *g, const nvd_solve_opts &o, int32_t k, int KT, size
         double us;
         int kt, cs;   // columns per tile (one kernel) or CTAs per cluster
     };
-    std::vector<Form> forms;
+    Form forms[5];
+    int nf = 0;
+    auto rank = [&](const Form &f) {   // fastest first, the earlier of equals before the later
+        int i = nf++;
+        for (; i > 0 && f.us < forms[i - 1].us; --i) forms[i] = forms[i - 1];
+        forms[i] = f;
+    };
     Form c{0.0, 0, 0};
     NVD_TRY(cluster_estimate(g, k, &c.cs, &c.us));
-    if (c.cs) forms.push_back(c);
+    if (c.cs) rank(c);
     // a call without a final synchronisation has nobody to report a wait that gave up to
     if (g->nseg == 1 && !(o.flags & NVD_SOLVE_NO_SYNC))
         for (int kt : {1, 4, 8, 16}) {
             if (kt > KT && kt > 1) break;
-            forms.push_back(Form{((k + kt - 1) / kt) * resident_iter_us(g->h_seg_end[0] - g->h_seg_begin[0], g->nnz, kt),
-                                 kt, 0});
+            rank(Form{((k + kt - 1) / kt) * resident_iter_us(g->h_seg_end[0] - g->h_seg_begin[0], g->nnz, kt), kt, 0});
         }
-    std::stable_sort(forms.begin(), forms.end(), [](const Form &u, const Form &v) { return u.us < v.us; });
     const double tiles = tiles_iter_us(g->n, g->nnz, KT, (k + KT - 1) / KT);
-    for (const Form &f : forms) {
-        if (!(f.us < tiles)) break;
+    for (int i = 0; i < nf && forms[i].us < tiles; ++i) {
+        const Form &f = forms[i];
         if (f.cs) NVD_TRY(unless_oom(cluster_plan_get(g, f.cs, cluster)));
         else NVD_TRY(unless_oom(resident_plan_for(g, f.kt, resident)));
         if (*cluster || *resident) break;
