@@ -400,23 +400,7 @@ __global__ void __launch_bounds__(CL_MAX_NT, 1) k_cluster_pcg(const __grid_const
             const int it = st.iters + 1;
             st.iters = it;
             st.rr = rr;
-            // the d^2 stop of FinBeta (kernels.cuh)
-            bool d2_done = false;
-            if (a.d2stop > 0.0) {
-                const double t = st.alpha * st.rho;
-                const double sum = st.hs_sum + t;
-                st.hs_sum = sum;
-                bool ok = it > d2_window() && t > 0.0;
-                double qm = 0.0, nxt = t;
-                for (int k = 0; k < d2_window(); ++k) {
-                    const double prev = st.hist[k];
-                    ok = ok && prev > 0.0;
-                    if (prev > 0.0) qm = fmax(qm, nxt / prev);
-                    st.hist[k] = nxt;
-                    nxt = prev;
-                }
-                d2_done = ok && qm < 0.95 && t * qm <= d2_safety() * a.d2stop * sum * (1.0 - qm);
-            }
+            const bool d2_done = a.d2stop > 0.0 && d2_settled(it, st.alpha * st.rho, a.d2stop, st.hs_sum, st.hist);
             int end = -1;
             if (st.status == NVD_ERR_NUMERIC || !finite(rr) || !finite(rho_new)) end = NVD_ERR_NUMERIC;
             else if (rr <= st.stop || d2_done) end = NVD_OK;

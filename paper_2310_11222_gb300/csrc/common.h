@@ -32,6 +32,23 @@ constexpr int sp_span_max() { return 2048; }
 // traces of ER, BA, WS and SBM graphs of mean degree 2..32, paths and cycles).
 constexpr int d2_window() { return 6; }
 constexpr double d2_safety() { return 0.03; }
+// The d^2 stop at step `it` of one pair, whose d^2 rose by t (FinBeta, kernels.cuh, explains it):
+// adds t to `sum`, shifts it into the last increments h (newest first), and says whether the
+// extrapolated gap is within d2stop of the sum.
+__device__ __forceinline__ bool d2_settled(int it, double t, double d2stop, double &sum, double *h) {
+    const double total = sum + t;
+    sum = total;
+    bool ok = it > d2_window() && t > 0.0;
+    double q = 0.0, nxt = t;
+    for (int w = 0; w < d2_window(); ++w) {
+        const double prev = h[w];
+        ok = ok && prev > 0.0;
+        if (prev > 0.0) q = fmax(q, nxt / prev);
+        h[w] = nxt;
+        nxt = prev;
+    }
+    return ok && q < 0.95 && t * q <= d2_safety() * d2stop * total * (1.0 - q);
+}
 // Columns one lane owns (16-byte vectors where the row is that wide), lanes per
 // row, and rows per slice (one row per lane group of a warp).
 constexpr int sp_vec(int KT, int szv) { return KT * szv >= 16 ? 16 / szv : KT; }

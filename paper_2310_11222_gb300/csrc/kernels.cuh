@@ -574,23 +574,8 @@ struct FinBeta {
         c.iters[i] = it;
         const double rho_new = s[0], rr = s[1];
         c.rr[i] = rr;
-        bool d2_done = false;
-        if (c.d2stop > 0.0) {
-            double *h = c.hs_hist + i * d2_window();   // t_{k-1}, t_{k-2}, ...
-            const double t = c.alpha[i] * c.rho[i];
-            const double sum = c.hs_sum[i] + t;
-            c.hs_sum[i] = sum;
-            bool ok = it > d2_window() && t > 0.0;
-            double q = 0.0, nxt = t;
-            for (int w = 0; w < d2_window(); ++w) {
-                const double prev = h[w];
-                ok = ok && prev > 0.0;
-                if (prev > 0.0) q = fmax(q, nxt / prev);
-                h[w] = nxt;
-                nxt = prev;
-            }
-            d2_done = ok && q < 0.95 && t * q <= d2_safety() * c.d2stop * sum * (1.0 - q);
-        }
+        const bool d2_done = c.d2stop > 0.0 && d2_settled(it, c.alpha[i] * c.rho[i], c.d2stop, c.hs_sum[i],
+                                                          c.hs_hist + i * d2_window());
         int st = -1;
         if (c.status[i] == NVD_ERR_NUMERIC || !isfinite(rr) || !isfinite(rho_new))
             st = NVD_ERR_NUMERIC;

@@ -371,23 +371,7 @@ __global__ void __launch_bounds__(RS_NT, 1) k_resident_pcg(const __grid_constant
                     const int it = st.iters[c] + 1;
                     st.iters[c] = it;
                     st.rr[c] = rr;
-                    // the d^2 stop of FinBeta (kernels.cuh)
-                    bool d2_done = false;
-                    if (a.d2stop > 0.0) {
-                        const double t = st.alpha[c] * st.rho[c];
-                        const double sum = st.hs_sum[c] + t;
-                        st.hs_sum[c] = sum;
-                        bool ok = it > d2_window() && t > 0.0;
-                        double qm = 0.0, nxt = t;
-                        for (int k = 0; k < d2_window(); ++k) {
-                            const double prev = st.hist[c][k];
-                            ok = ok && prev > 0.0;
-                            if (prev > 0.0) qm = fmax(qm, nxt / prev);
-                            st.hist[c][k] = nxt;
-                            nxt = prev;
-                        }
-                        d2_done = ok && qm < 0.95 && t * qm <= d2_safety() * a.d2stop * sum * (1.0 - qm);
-                    }
+                    const bool d2_done = a.d2stop > 0.0 && d2_settled(it, st.alpha[c] * st.rho[c], a.d2stop, st.hs_sum[c], st.hist[c]);
                     int end = -1;
                     if (st.status[c] == NVD_ERR_NUMERIC || !finite(rr) || !finite(rho_new)) end = NVD_ERR_NUMERIC;
                     else if (rr <= a.rtol2 * st.rr0[c] || d2_done) end = NVD_OK;
