@@ -437,7 +437,8 @@ struct ResidentPlan {
     size_t smem = 0;
     int64_t n_slots = 0;
     // two allocations and one copy: with one each, a new graph's first call took 10 ms instead
-    // of 4 at 100,000 nodes (the rest of that was a comparison sort)
+    // of 4 at 100,000 nodes (the rest of that was a comparison sort; 2.6 since only the plan that
+    // is used is built)
     DevBuf meta, data;
     RsCta *ctas = nullptr;
     Item *items = nullptr;
